@@ -157,9 +157,9 @@ typedef struct rb_update_params {
                                alternatives and pass the fastest; the results do not change):
                                bits 0-1 the rasteriser's work mapping, 1 = warps along the ray tubes,
                                2 = warps across them (rule: along from tubes of 4 pixels at the ring);
-                               bits 2-3 the tensor-core adjoint, 1 = CTA pairs (cta_group::2 MMAs),
-                               2 = one CTA per pixel tile (the rule); other bits 0; a field of 3
-                               returns RB_ERR_ARG */
+                               bits 2-3 the tensor-core adjoint, 1 and 2 accepted from callers that
+                               chose between two forms of it: there is one, one CTA per pixel tile;
+                               other bits 0; a field of 3 returns RB_ERR_ARG */
     void* stage_events;     /* NULL, or a caller-created array of 2 * RB_STAGE_COUNT cudaEvent_t:
                                events [2s] and [2s+1] are recorded on the stream before and after
                                stage s (no events are created or destroyed by the library) */

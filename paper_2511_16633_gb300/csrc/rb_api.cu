@@ -303,12 +303,7 @@ rb_status gradient_stages(const GeoDev& G, const FreqSet& F, const Ws& W, float*
     RB_CU(launch_link(G, c, ends, F, R, linked, s2));
     RB_CU(launch_residual_keys(G, n_freq, (const float2*)p_obs, R, linked, keys, cnt, W.at<void>(W.L.sel), s2));
     RB_CU(launch_outlier_select(n_freq * ne2, params->outlier_frac, keys, cnt, wts, W.at<void>(W.L.sel), s2));
-    if (tc) {
-        const size_t img = tc_b_images_bytes(G.n_elem);
-        for (int w = 0; w < n_freq; ++w)
-            RB_CU(launch_prep_b(G.n_elem, R + (size_t)w * ne2, wts + (size_t)w * ne2, W.at<char>(W.L.tcimg) + w * img,
-                                s2));
-    }
+    if (tc) RB_CU(launch_prep_b(G.n_elem, n_freq, R, wts, W.at<void>(W.L.tcimg), s2));
     RB_CU(mark2(RB_STAGE_LINK, 1));
     RB_CU(cudaEventRecord(ss->join, s2));
     // main branch: rasteriser and resolve (in launch_trace; on the mixed path with the
@@ -320,8 +315,7 @@ rb_status gradient_stages(const GeoDev& G, const FreqSet& F, const Ws& W, float*
     RB_CU(mark(RB_STAGE_ADJOINT, 0));
     if (tc) {
         RB_CU(launch_adjoint_tc(G, W.at<void>(W.L.aimg), F, W.at<void>(W.L.tcimg), W.at<float2>(W.L.gscr), tc_ctas(),
-                                nullptr, nullptr, W.at<float>(W.L.gsum), W.at<float>(W.L.hsum), cnt, s,
-                                (params->tune >> 2) & 3));
+                                nullptr, nullptr, W.at<float>(W.L.gsum), W.at<float>(W.L.hsum), cnt, s));
     } else {
         RB_CU(launch_adjoint_simt(G, tables, c, F, R, wts, nullptr, nullptr, W.at<float>(W.L.gsum),
                                   W.at<float>(W.L.hsum), cnt, s));
@@ -363,9 +357,9 @@ size_t rb_ws_layout(const rb_geometry* g, int n_freq, rb_precision prec, WsLayou
     L->part = o; o = align256(o + (size_t)(RB_MAX_FREQ + 2) * 256 * 8);
     L->fwd = o; o = align256(o + (tcp ? 0 : (size_t)rb_fwd_chunks_for((int)npix) * ne * ne * 8));
     L->tcimg = o; o = align256(o + (tcp ? (size_t)n_freq * tc_b_images_bytes(g->n_elem) : 0));
-    // exact G per persistent CTA, then its |G|^2 A slices (bf16 hi and lo), then (Re g, H)
+    // two sets of |G|^2 A slices (bf16 hi and lo) per persistent CTA, then (Re g, H)
     // of each frequency of the set for the adjoint's sums over the set
-    L->gscr = o; o = align256(o + (tcp ? (size_t)RB_TC_MAX_CTAS * ne * 128 * (8 + 4) + nf * npix * 8 : 0));
+    L->gscr = o; o = align256(o + (tcp ? (size_t)RB_TC_MAX_CTAS * ne * 128 * 8 + nf * npix * 8 : 0));
     // two of them on the update path: one frequency's reduce runs beside the next one's forward
     L->tcfwd = o; o = align256(o + (tcp ? 2 * align256(tc_forward_partial_bytes(g->n_elem, RB_TC_MAX_CTAS)) : 0));
     L->aimg = o; o = align256(o + (tcp ? (size_t)n_freq * tc_aimage_elems(g->n_elem, (int)npix) * 2 : 0));
@@ -545,7 +539,7 @@ rb_status rb_born_adjoint(const rb_geometry* geom, const rb_cell* tables, const 
     RB_CU(launch_elem_positions(G, exy, s));
     if (prec == RB_PREC_BF16X3) {
         RB_CU(cudaMemsetAsync(cnt, 0, CNT_N * 4, s));
-        RB_CU(launch_prep_b(G.n_elem, (const float2*)resid, w, W.at<void>(W.L.tcimg), s));
+        RB_CU(launch_prep_b(G.n_elem, 1, (const float2*)resid, w, W.at<void>(W.L.tcimg), s));
         RB_CU(launch_tables_images(G, tables, c, F, W.at<void>(W.L.aimg), s));
         RB_CU(launch_adjoint_tc(G, W.at<void>(W.L.aimg), F, W.at<void>(W.L.tcimg), W.at<float2>(W.L.gscr), tc_ctas(),
                                 (float2*)g_out, hdiag_out, nullptr, nullptr, cnt, s));
@@ -654,7 +648,6 @@ rb_status rb_cg_update(const rb_geometry* geom, float* c_inout, const float* alp
     // the residuals are consumed by the gradient: their buffer holds B_w p from here on
     float2* d = W.at<float2>(W.L.pray);
     const bool tc = prec == RB_PREC_BF16X3;
-    const size_t img = tc_b_images_bytes(G.n_elem);
     const int nch = rb_fwd_chunks_for(G.npix);
     RB_CU(mark(RB_STAGE_DIRECTION, 0));
     RB_CU(launch_cg_init(G, gsum, hsum, precond, x, r, p, part, dbl, params->eps_rel, s));
@@ -668,7 +661,6 @@ rb_status rb_cg_update(const rb_geometry* geom, float* c_inout, const float* alp
                 RB_CU(launch_forward_tc(G, W.at<char>(W.L.aimg) + (size_t)w * tc_aimage_elems(G.n_elem, G.npix) * 2,
                                         F.f[w], p, W.at<float>(W.L.tcfwd), tc_ctas(), dw, wts + (size_t)w * ne2,
                                         part + (size_t)w * 256, cnt, s));
-                RB_CU(launch_prep_b(G.n_elem, dw, wts + (size_t)w * ne2, W.at<char>(W.L.tcimg) + w * img, s));
             } else {
                 RB_CU(launch_forward_simt(G, tables, c_inout, F.f[w], p, W.at<float2>(W.L.fwd), nch, s));
                 RB_CU(launch_forward_reduce(G, F.f[w], W.at<float2>(W.L.fwd), nch, dw, wts + (size_t)w * ne2,
@@ -678,8 +670,9 @@ rb_status rb_cg_update(const rb_geometry* geom, float* c_inout, const float* alp
         RB_CU(launch_sum_partials(part, n_freq * 256, dbl, DBL_CG_PAP + k, 1.0, 0, s));
         // q = sum_w Re B_w^H W B_w p
         if (tc) {
+            RB_CU(launch_prep_b(G.n_elem, n_freq, d, wts, W.at<void>(W.L.tcimg), s));
             RB_CU(launch_adjoint_tc(G, W.at<void>(W.L.aimg), F, W.at<void>(W.L.tcimg), W.at<float2>(W.L.gscr),
-                                    tc_ctas(), nullptr, nullptr, q, nullptr, cnt, s, (params->tune >> 2) & 3));
+                                    tc_ctas(), nullptr, nullptr, q, nullptr, cnt, s));
         } else {
             RB_CU(launch_adjoint_simt(G, tables, c_inout, F, d, wts, nullptr, nullptr, q, nullptr, cnt, s));
         }

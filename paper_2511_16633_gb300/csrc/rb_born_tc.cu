@@ -1,18 +1,19 @@
 // Tensor-core (tcgen05, BF16 x3 split products, FP32 accumulation in TMEM) Born
-// adjoint and Gauss-Newton Hessian diagonal with fused Green's-function synthesis.
+// adjoint and Gauss-Newton Hessian diagonal, and Born forward.
 //
-// Per frequency w and tile of 128 pixels x (the MMA's M rows):
-//   U[x][e']  = sum_k' A[x][k'] B[e'][k'],   k' = 2r + {0: Re, 1: Im}
-//     A[x][2r] = Re G_r(x), A[x][2r+1] = -Im G_r(x)           (conj G, synthesised)
-//     e' < n:  B = (Re S[e][r], -Im S[e][r])  ->  U = Re (S conj G)[e]
-//     e' >= n: B = (Im S[e][r],  Re S[e][r])  ->  U = Im (S conj G)[e]
-//   g(x) = w^2 sum_e conj(G_e(x)) U_e(x),  S = W o R
-//   V[x][e]   = sum_r |G_r(x)|^2 W[e][r],    H(x) = w^4 sum_e |G_e(x)|^2 V[x][e]
+// Adjoint, per frequency w and tile of 128 pixels x (the MMA's M rows).  Both sums are
+// symmetric in emitter and receiver, so only r <= e is multiplied out:
+//   g(x) = w^2 sum_e conj(G_e(x)) U_e(x),   U_e = sum_{r <= e} T[e][r] conj(G_r),  S = W o R
+//   H(x) = w^4 sum_e |G_e(x)|^2 V_e(x),     V_e = sum_{r <= e} Y[e][r] |G_r|^2
+// with T = S + S^T and Y = W + W^T below the block diagonal (blocks of 8 elements for T,
+// of 32 for Y) and T = S, Y = W inside the diagonal blocks: half the products of the full
+// sums, the same value.
+//   U[x][e'] = sum_k' A[x][k'] B[e'][k'],   k' = 2r + {0: Re, 1: Im},  A = (Re G_r, -Im G_r)
+//   e' = 16 (e / 8) + e % 8:      B = (Re T[e][r], -Im T[e][r])  ->  Re U_e
+//   e' = 16 (e / 8) + 8 + e % 8:  B = (Im T[e][r],  Re T[e][r])  ->  Im U_e
 // Each operand is split into bf16 hi + lo and the products hi*hi + hi*lo + lo*hi
-// (U) or hi*W + lo*W (V, W is exact in bf16) accumulate in fp32 in TMEM, which
-// keeps ~2^-16 relative accuracy per product.  The epilogue uses the exact fp32
-// G values, kept per CTA in a small L2-resident scratch while the K loop streams
-// bf16 chunks of A through shared memory.
+// (U) or hi*Y + lo*Y (V, Y in {0, 1, 2} is exact in bf16) accumulate in fp32 in TMEM, which
+// keeps ~2^-16 relative accuracy per product.
 #include <cuda.h>
 
 #include "rb_internal.cuh"
@@ -23,72 +24,158 @@ namespace {
 constexpr int TP = RB_TP;               // pixels per tile = MMA M
 constexpr uint32_t kMaxTries = 1u << 22; // mbarrier polls before giving up (each poll suspends briefly)
 
-// ---------------------------------------------------------------------------
-// B operand images for one frequency, in K slices of 16 (one pipeline stage each)
-// in the core-matrix layout of rb_tc.cuh (tile16_offset).
-//   bu: [ks = 2n/16][hi|lo][2n rows x 16]   (2n rows = e', K = 2n)
-//   bw: [ks = n/32][n rows x 32]            (W, exact; K = 32 slices, chunk_offset)
-// ---------------------------------------------------------------------------
-__global__ void k_prep_b(int n, const float2* __restrict__ R, const uint8_t* __restrict__ W,
-                         __nv_bfloat16* __restrict__ bu, __nv_bfloat16* __restrict__ bw) {
-    const int n2 = 2 * n;
-    const size_t img_u = (size_t)n2 * 16;  // bf16 per hi or lo image of one slice
-    const long long total_u = (long long)n2 * n2;
-    for (long long j = blockIdx.x * (long long)blockDim.x + threadIdx.x; j < total_u;
-         j += (long long)gridDim.x * blockDim.x) {
-        const int ep = (int)(j / n2), kp = (int)(j % n2);
-        const int r = kp >> 1, part = kp & 1;
-        // rows e' in N-blocks of nb columns (the adjoint's MMA width), each holding the
-        // Re U rows then the Im U rows of nb / 2 consecutive elements; a pass of the
-        // adjoint takes ne2 = 2 min(n, 256) rows in one or two N-blocks
-        const int ne2 = n2 < 512 ? n2 : 512;
-        const int nb = ne2 > 256 ? ne2 / 2 : ne2, eb = nb / 2;
-        const int blk = ep / nb, w = ep % nb;
-        const int e = blk * eb + w % eb, im = w / eb;
-        float2 s = make_float2(0.f, 0.f);
-        if (W[(size_t)e * n + r]) s = R[(size_t)e * n + r];
-        float v;
-        if (im == 0) v = part == 0 ? s.x : -s.y;
-        else v = part == 0 ? s.y : s.x;
-        __nv_bfloat16 hi, lo;
-        tc::split_bf16(v, hi, lo);
-        const int ks = kp >> 4, kk = kp & 15;
-        const size_t base = (size_t)ks * 2 * img_u;
-        const uint32_t off = tc::tile16_offset((uint32_t)ep, (uint32_t)kk) / 2;
-        bu[base + off] = hi;
-        bu[base + img_u + off] = lo;
+// The adjoint takes the elements e in passes of ne = min(n, 256) (the accumulators of one
+// pass fit TMEM); pass q covers e in [q ne, (q + 1) ne) and sums over r < (q + 1) ne.  Its
+// K slices of 8 elements r: slices j < q ne / 8 lie below the block diagonal and feed all
+// 2 ne columns; slice d = j - q ne / 8 on the diagonal feeds the columns from 16 d on.
+// Likewise the V slices of 32 elements r and the columns from 32 d on.
+struct AdjShape {
+    int n, ne, ge, gv;                  // elements; per pass: elements, groups of 8, blocks of 32
+    __host__ __device__ explicit AdjShape(int n_) : n(n_), ne(n_ < 256 ? n_ : 256), ge(ne / 8), gv(ne / 32) {}
+    // rows e' of U slice j (rows e of V slice i) in pass q
+    __host__ __device__ int u_rows(int q, int j) const { return 2 * ne - 16 * (j > q * ge ? j - q * ge : 0); }
+    __host__ __device__ int v_rows(int q, int i) const { return ne - 32 * (i > q * gv ? i - q * gv : 0); }
+    // bytes of the images before slice j of pass q (64 bytes a row: U hi and lo of 16 K values, V 32 K values)
+    __host__ __device__ size_t u_off(int q, int j) const {
+        size_t rows = 0;
+        for (int p = 0; p < q; ++p) rows += (size_t)p * ge * 2 * ne + (size_t)ge * 2 * ne - 8u * (size_t)ge * (ge - 1);
+        const int full = j < q * ge ? j : q * ge, d = j - full;
+        rows += (size_t)full * 2 * ne + (size_t)d * 2 * ne - (d > 0 ? 8u * (size_t)d * (d - 1) : 0u);
+        return rows * 64;
     }
-    const long long total_w = (long long)n * n;
-    const size_t img_w = (size_t)n * 32;
-    for (long long j = blockIdx.x * (long long)blockDim.x + threadIdx.x; j < total_w;
-         j += (long long)gridDim.x * blockDim.x) {
-        const int e = (int)(j / n), r = (int)(j % n);
-        const int ks = r >> 5, kk = r & 31;
-        bw[(size_t)ks * img_w + tc::chunk_offset((uint32_t)e, (uint32_t)kk) / 2] =
-            __float2bfloat16_rn(W[(size_t)e * n + r] ? 1.f : 0.f);
+    __host__ __device__ size_t v_off(int q, int i) const {
+        size_t rows = 0;
+        for (int p = 0; p < q; ++p) rows += (size_t)p * gv * ne + (size_t)gv * ne - 16u * (size_t)gv * (gv - 1);
+        const int full = i < q * gv ? i : q * gv, d = i - full;
+        rows += (size_t)full * ne + (size_t)d * ne - (d > 0 ? 16u * (size_t)d * (d - 1) : 0u);
+        return rows * 64;
+    }
+};
+
+// ---------------------------------------------------------------------------
+// B operand images of every frequency of a set, in the core-matrix layouts of rb_tc.cuh,
+// each slice holding the rows its pass multiplies and the slices packed in pass order:
+//   bu: [pass, slice of 8 elements r][hi|lo][rows e' x 16]   (tile16_offset)
+//   bw: [pass, slice of 32 elements r][rows e x 32]           (chunk_offset)
+// CTA (slice, frequency); a thread takes one row's 4 (U) or 8 (V) elements r and writes
+// its 16-byte core rows: 256 elements, 4 frequencies in one launch (four launches of
+// 6.5 us each, one bf16 per store, before).
+// ---------------------------------------------------------------------------
+__global__ void __launch_bounds__(128) k_prep_b(int n, const float2* __restrict__ Rs, const uint8_t* __restrict__ Ws,
+                                                unsigned char* __restrict__ img, size_t img_stride, size_t w_off) {
+    const AdjShape sh(n);
+    const float2* R = Rs + (size_t)blockIdx.y * n * n;
+    const uint8_t* W = Ws + (size_t)blockIdx.y * n * n;
+    unsigned char* out = img + (size_t)blockIdx.y * img_stride;
+    const int npass = n / sh.ne, nu = sh.ge * npass * (npass + 1) / 2;
+    const bool is_v = (int)blockIdx.x >= nu;
+    const int per = is_v ? sh.gv : sh.ge;   // slices added per pass
+    int j = (int)blockIdx.x - (is_v ? nu : 0), q = 0;
+    while (j >= per * (q + 1)) j -= per * ++q;
+    if (!is_v) {
+        const int rows = sh.u_rows(q, j), cnt = rows / 2, e0 = (q + 1) * sh.ne - cnt;
+        unsigned char* dst = out + sh.u_off(q, j);
+        for (int idx = threadIdx.x; idx < 2 * cnt; idx += blockDim.x) {
+            const int el = idx % cnt, kc = idx / cnt, e = e0 + el;
+            uint32_t rh[4], rl[4], ih[4], il[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int r = 8 * j + 4 * kc + k;
+                float2 s = make_float2(0.f, 0.f);
+                if (W[(size_t)e * n + r]) s = R[(size_t)e * n + r];
+                if ((e >> 3) > j && W[(size_t)r * n + e]) {
+                    const float2 t = R[(size_t)r * n + e];
+                    s.x += t.x;
+                    s.y += t.y;
+                }
+                __nv_bfloat16 xh, xl, yh, yl;
+                tc::split_bf16(s.x, xh, xl);
+                tc::split_bf16(s.y, yh, yl);
+                rh[k] = bf16_pack2(xh, __hneg(yh));
+                rl[k] = bf16_pack2(xl, __hneg(yl));
+                ih[k] = bf16_pack2(yh, xh);
+                il[k] = bf16_pack2(yl, xl);
+            }
+            const uint32_t row = 16u * (uint32_t)(el >> 3) + (uint32_t)(el & 7);
+            const uint32_t o = tc::tile16_offset(row, 8u * (uint32_t)kc), lo = (uint32_t)rows * 32u;
+            *(uint4*)(dst + o) = make_uint4(rh[0], rh[1], rh[2], rh[3]);
+            *(uint4*)(dst + lo + o) = make_uint4(rl[0], rl[1], rl[2], rl[3]);
+            *(uint4*)(dst + o + tc::kRowGroupBytes16) = make_uint4(ih[0], ih[1], ih[2], ih[3]);
+            *(uint4*)(dst + lo + o + tc::kRowGroupBytes16) = make_uint4(il[0], il[1], il[2], il[3]);
+        }
+    } else {
+        const int rows = sh.v_rows(q, j), e0 = (q + 1) * sh.ne - rows;
+        unsigned char* dst = out + w_off + sh.v_off(q, j);
+        for (int idx = threadIdx.x; idx < 4 * rows; idx += blockDim.x) {
+            const int el = idx % rows, core = idx / rows, e = e0 + el;
+            uint32_t v[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                const int r = 32 * j + 8 * core + k;
+                v[k] = W[(size_t)e * n + r] ? 1u : 0u;
+                if ((e >> 5) > j && W[(size_t)r * n + e]) ++v[k];
+                v[k] = v[k] == 0u ? 0u : (v[k] == 1u ? 0x3f80u : 0x4000u);   // bf16 0, 1, 2
+            }
+            *(uint4*)(dst + tc::chunk_offset((uint32_t)el, 8u * (uint32_t)core)) =
+                make_uint4(v[0] | v[1] << 16, v[2] | v[3] << 16, v[4] | v[5] << 16, v[6] | v[7] << 16);
+        }
     }
 }
 
+constexpr int ADJ_MAX_ENT = 384;   // schedule entries of a pixel tile (372 for 1024 elements)
+constexpr int ADJ_MAX_WORK = 24;   // work records of a quad and pixel tile (six a pass)
+
+// One schedule entry (a pipeline stage): U slices j .. j + cnt - 1 or V slice j, and for a
+// diagonal one the diagonal index d = j - (first diagonal slice of the pass).
+struct AdjEnt {
+    uint32_t v;
+    static __host__ __device__ AdjEnt make(int j, int cnt, bool is_v, bool first, int d) {
+        return AdjEnt{(uint32_t)j | (uint32_t)cnt << 8 | (is_v ? 1u << 11 : 0u) | (first ? 1u << 12 : 0u) |
+                      (d >= 0 ? 1u << 16 | (uint32_t)d << 17 : 0u)};
+    }
+    __host__ __device__ uint32_t j() const { return v & 0xffu; }
+    __host__ __device__ uint32_t cnt() const { return (v >> 8) & 7u; }
+    __host__ __device__ bool is_v() const { return (v & (1u << 11)) != 0u; }
+    __host__ __device__ bool first() const { return (v & (1u << 12)) != 0u; }   // first entry of its pass
+    __host__ __device__ bool diag() const { return (v & (1u << 16)) != 0u; }
+    __host__ __device__ uint32_t d() const { return v >> 17; }                    // 0 below the diagonal
+};
+
+// One piece of a quad's work: U unit u (groups 2u, 2u + 1 of the pass) or V slice u.  a, b:
+// where the unit's two A slices (V: its stage, in a) are staged: stage ordinal (entry
+// number mod NST) | KB offset << 4 | arrivals per warp << 12 | full barrier (first group
+// of the entry) << 16; b = 0 when both slices are in one entry, whose second offset is
+// then in off2.
+struct AdjWork {
+    uint32_t x, a, b, off2;
+    __host__ __device__ uint32_t u() const { return x & 0xffu; }
+    __host__ __device__ uint32_t q() const { return (x >> 8) & 7u; }
+    __host__ __device__ bool is_v() const { return (x & (1u << 11)) != 0u; }
+    __host__ __device__ bool first() const { return (x & (1u << 12)) != 0u; }   // the quad's first of its pass
+    __host__ __device__ bool last() const { return (x & (1u << 13)) != 0u; }    // its last of the pass
+    __host__ __device__ bool low() const { return (x & (1u << 14)) != 0u; }     // its last unit in columns V takes over
+};
+
 struct TcArgs {
     GeoDev G;
-    FreqSet F;
     const __nv_bfloat16* aimg; // [n_freq][tiles][hi|lo][2n / 8 rows][1024] A image (layout: aimg_put4)
     size_t aimg_stride;        // bf16 elements per frequency
-    const __nv_bfloat16* bu;   // [n_freq][image]
-    const __nv_bfloat16* bw;   // [n_freq][image]
-    size_t bu_stride, bw_stride;  // bf16 elements per frequency
-    float2* gscr;              // [gridDim.x][n][TP] exact G per CTA
-    __nv_bfloat16* vimg;       // [gridDim.x][n / 32][hi|lo][TP x 32] |G|^2 A slices of the Hessian contraction
+    const unsigned char* bu;   // [n_freq][image]
+    const unsigned char* bw;   // [n_freq][image]
+    size_t b_stride;           // bytes per frequency
+    __nv_bfloat16* vimg;       // [gridDim.x][2][n / 32][hi|lo][TP x 32] |G|^2 A slices of the Hessian contraction
     float2* g_out;             // [n_freq][npix] or null
     float* h_out;              // [n_freq][npix] or null
-    float* gsum;               // [npix] or null (sum over w of Re g)
-    float* hsum;               // [npix] or null
     float2* fpart;             // [n_freq][npix] (Re g, H) of each frequency for k_adjoint_sums, or null
     uint32_t* counters;
-    int n_tiles;
-    uint32_t tmem_cols;
-    int n_e, npass;            // elements per pass (N of the MMAs: 2 n_e and n_e), passes = n / n_e
+    float w2[RB_MAX_FREQ], w4[RB_MAX_FREQ];
+    int n_freq, n_tiles;
     int want_h;                // the Hessian contraction is wanted (h_out or hsum set)
+    uint32_t tmem_cols, v_col; // TMEM columns; first column of V (U has columns 0 .. 2 ne - 1)
+    int low_groups;            // groups of U whose columns V overwrites (0: V has columns of its own)
+    int n_ent, n_work[4];
+    AdjEnt ent[ADJ_MAX_ENT];   // the slices of one (tile, frequency), in order
+    AdjWork work[4][ADJ_MAX_WORK];   // each quad's part, in the same order
 };
 
 }  // namespace
@@ -96,8 +183,8 @@ struct TcArgs {
 namespace {
 
 // Pipeline shapes of the tensor-core kernels.
-constexpr int NPROD = 512;                   // adjoint producer threads: four per pixel row
-constexpr int NTHR_A = NPROD + 64;           // + MMA warp + B-loader warp
+constexpr int NPROD = 512;                   // adjoint epilogue threads: four quads of 128 (thread = pixel)
+constexpr int NTHR_A = NPROD + 64;           // + MMA warp + loader warp
 constexpr int NPROD_F = 256;                 // forward producer threads: two per A row
 constexpr int NTHR_F = NPROD_F + 64;
 constexpr int NST = 5;                       // pipeline stages
@@ -110,60 +197,12 @@ __device__ __forceinline__ uint32_t pack2(__nv_bfloat16 a, __nv_bfloat16 b) {
     return (uint32_t)__bfloat16_as_ushort(a) | ((uint32_t)__bfloat16_as_ushort(b) << 16);
 }
 
-// |G|^2 of elements e .. e + 7 (e a multiple of 8) at pixel p, hi and lo planes, from the
-// tile's V A slices (written by consume_u; K = 32 slices in the chunk_offset layout, so
-// the 8 values of a plane are 16 contiguous bytes): half the bytes of reading G back.
-__device__ __forceinline__ void g2_load(const __nv_bfloat16* vimg, int e, uint32_t p, uint4 (&q)[2]) {
-    const __nv_bfloat16* vs = vimg + (size_t)(e >> 5) * (2 * TP * 32);
-    const uint32_t vo = tc::chunk_offset(p, (uint32_t)(e & 31)) / 2;
-    q[0] = *(const uint4*)(vs + vo);
-    q[1] = *(const uint4*)(vs + TP * 32 + vo);
+// The two bf16 halves of a packed word, hi + lo parts added (exact: lo is below hi's ulp).
+__device__ __forceinline__ float sum_lo16(uint32_t h, uint32_t l) {
+    return __uint_as_float(h << 16) + __uint_as_float(l << 16);
 }
-
-// hh += sum_i |G_i|^2 V_i over a chunk of 8 elements: V from TMEM (8 columns at taddr),
-// |G|^2 = hi + lo (the values the V MMAs used).
-__device__ __forceinline__ void h_chunk(uint32_t taddr, const uint4 (&q)[2], float& hh) {
-    float v[8];
-    tc::tmem_ld8(taddr, v);
-    const uint32_t wh[4] = {q[0].x, q[0].y, q[0].z, q[0].w}, wl[4] = {q[1].x, q[1].y, q[1].z, q[1].w};
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const float g0 = __bfloat162float(__ushort_as_bfloat16((unsigned short)(wh[i] & 0xffffu))) +
-                         __bfloat162float(__ushort_as_bfloat16((unsigned short)(wl[i] & 0xffffu)));
-        const float g1 = __bfloat162float(__ushort_as_bfloat16((unsigned short)(wh[i] >> 16))) +
-                         __bfloat162float(__ushort_as_bfloat16((unsigned short)(wl[i] >> 16)));
-        hh = fmaf(g0, v[2 * i], hh);
-        hh = fmaf(g1, v[2 * i + 1], hh);
-    }
-}
-
-// Producer work of one U slice (8 elements, K' = 16) for thread (p, h), h < 4: the
-// A slice in shared memory (two rows of the A image, layout of aimg_put4) holds, at
-// K' positions 4h .. 4h + 3 of row p, the bf16
-// hi / lo parts of (Re G, -Im G) of elements r0 + 2h + j (j < 2).  Their sums give
-// G to ~2^-17 relative for the epilogue (gs), and |G|^2 (hi / lo) goes to the V
-// slice r0 / 16 of this CTA.
-__device__ __forceinline__ void consume_u(int r0, uint32_t p, uint32_t h, const unsigned char* a_hi,
-                                          const unsigned char* a_lo, float2* gs, __nv_bfloat16* vimg, bool want_h) {
-    // A slice = two image rows (K cores) of 2 KB: K core h / 2, pixel core p / 8, row p % 8
-    const uint32_t off = (h >> 1) * 2048u + (p >> 3) * 128u + (p & 7u) * 16u + 8u * (h & 1u);
-    const uint2 wh = *(const uint2*)(a_hi + off), wl = *(const uint2*)(a_lo + off);
-    const uint32_t hw[2] = {wh.x, wh.y}, lw[2] = {wl.x, wl.y};
-    __nv_bfloat16 vh[2], vl[2];
-#pragma unroll
-    for (int j = 0; j < 2; ++j) {
-        const float re = __bfloat162float(__ushort_as_bfloat16((unsigned short)(hw[j] & 0xffffu))) +
-                         __bfloat162float(__ushort_as_bfloat16((unsigned short)(lw[j] & 0xffffu)));
-        const float mim = __bfloat162float(__ushort_as_bfloat16((unsigned short)(hw[j] >> 16))) +
-                          __bfloat162float(__ushort_as_bfloat16((unsigned short)(lw[j] >> 16)));
-        gs[(size_t)(r0 + 2 * (int)h + j) * TP + p] = make_float2(re, -mim);
-        tc::split_bf16(re * re + mim * mim, vh[j], vl[j]);
-    }
-    if (!want_h) return;
-    __nv_bfloat16* vs = vimg + (size_t)(r0 >> 5) * (2 * TP * 32);
-    const uint32_t voff = tc::chunk_offset(p, (uint32_t)(r0 & 31) + 2u * h) / 2;
-    *(uint32_t*)(vs + voff) = pack2(vh[0], vh[1]);
-    *(uint32_t*)(vs + TP * 32 + voff) = pack2(vl[0], vl[1]);
+__device__ __forceinline__ float sum_hi16(uint32_t h, uint32_t l) {
+    return __uint_as_float(h & 0xffff0000u) + __uint_as_float(l & 0xffff0000u);
 }
 
 // ---------------------------------------------------------------------------
@@ -215,56 +254,70 @@ __global__ void __launch_bounds__(256) k_tables_images(GeoDev G, const rb_cell* 
 }
 
 // ---------------------------------------------------------------------------
-// Adjoint kernel: warp-specialised, NST-stage pipeline of K = 16 slices.
-//   warps 0..15 producers: from each U slice's A (in shared memory, items of 8
-//               pixels x 4 K quarters per warp) they keep G for the epilogue (gs)
-//               and write the |G|^2 A slices of V; then the epilogues (TMEM ->
-//               registers; thread = pixel p = tid % 128, the TMEM lane, and quarter
-//               h = tid / 128 of the elements);
-//   warp 16     MMA issuer (lane 0): waits for a stage, issues its MMAs and
-//               commits their completion to the stage's "empty" barrier;
-//   warp 17     loader (lane 0): bulk-copies A and B of each slice (U: the A image
-//               and S; V: the |G|^2 slices and W) into a stage as soon as the
-//               stage's previous contents have been used.
-// Per (tile, frequency, pass over the elements) the slice sequence is U (2n / 16
-// slices of K = 16) then, when the Hessian diagonal is wanted, V (n / 32 slices of
-// K = 32); a pass covers 256 elements of e (all of them up to 256 elements), the
-// contractions always run over all of r.
-// Barriers: full[s] (bulk-copy bytes), empty[s] (the MMAs that read stage s done,
-// plus 16 producer-warp arrivals: A read), acc_full (last MMA of a phase done),
-// acc_empty (16 producer-warp arrivals: the epilogue has read the accumulator),
-// vready (16 producer-warp arrivals: the |G|^2 slices of this tile are written),
-// drain (MMA completion on the error path).  Every wait is bounded; a timeout
-// raises a shared flag that ends all loops.
+// Adjoint kernel: warp-specialised, NST-stage pipeline of 40 KB stages.
+//   warps 0..15 four epilogue quads of four warps (thread = pixel p = tid % 128 = the TMEM
+//               lane): quad u % 4 takes diagonal unit u (16 elements, two U slices).  It
+//               reads G of the unit from the staged A slices, writes the unit's |G|^2 (hi /
+//               lo) to the V slice in global scratch, and, once the MMAs of its second slice
+//               are complete, adds conj(G_e) U_e of the unit's 32 TMEM columns to its
+//               pixel's g: the columns of a unit get their last contribution from its own
+//               slices, so the epilogue follows the MMAs through the tile instead of
+//               waiting for its end, and G comes from slices that are in shared memory
+//               anyway.  V slices alike (quad dv % 4, 32 columns, |G|^2 from the stage).
+//   warp 16     MMA issuer: waits for a stage, issues its MMAs and commits their completion
+//               to the stage's "empty" barrier and to the diagonal units' own;
+//   warp 17     loader: bulk-copies A and B of the slices of a stage (U: the A image and T;
+//               V: the |G|^2 slices and Y) as soon as it is free.
+// The slice order of a (tile, frequency) is the schedule of adj_schedule(): the U slices
+// with r ascending, as many of the last, short ones to a stage as fit it, and the V slices
+// among them, each behind the U groups whose |G|^2 it reads and whose columns it takes.
+// Barriers: full_u[d] / full_v[dv] (bulk-copy bytes of an entry on the diagonal, d its
+// first group) and acc_u[u] / acc_v[dv] (MMAs complete), each used once per pass with the
+// pass's parity, so that a quad waits only for its own slices (a schedule has at least NST
+// entries, so no barrier can complete twice before its readers, without whom the stage is
+// not free, have seen it); full[s] (the slices below the diagonal, which only the issuer
+// waits for); empty[s] (the stage's MMAs, and 48 arrivals of the quads that read it, or of
+// the issuer where none does), acc_low (16 warp arrivals: the U columns that V takes over
+// are read), acc_empty (16 warp arrivals: every column of the pass is read), vready[dv] (8
+// warp arrivals: the |G|^2 slice is written), drain (MMA completion on the error path).
+// Every wait is bounded; a timeout raises a shared flag that ends all loops.
+//
+// What bounds it: shared-memory traffic first.  Per (tile, frequency) of 256 elements the
+// MMAs need 15 k cycles, and the stages' writes (0.98 MB), the MMAs' operand reads and the
+// quads' reads come to about 3 MB, 24 k cycles at 128 B a cycle (the full sums: 29 k cycles
+// of MMAs and 4.6 MB).  The rest was instruction latency of the two issuing warps: one
+// barrier wait per stage, polled ahead, and schedules worked out on the host keep it down.
 // ---------------------------------------------------------------------------
-// MULTI: more than one pass over the elements (rings above 256 elements, passes of 256);
-// the one-pass kernel is compiled without the pass bookkeeping.
-template <bool MULTI>
-__global__ void __launch_bounds__(NTHR_A, 1) k_adjoint_tc(TcArgs A) {
+__global__ void __launch_bounds__(NTHR_A, 1) k_adjoint_tc(const __grid_constant__ TcArgs A) {
     extern __shared__ __align__(1024) unsigned char smem[];
-    __shared__ uint64_t s_full[NST], s_empty[NST], s_acc_full, s_acc_empty, s_acc_low, s_vready, s_drain;
+    __shared__ uint64_t s_full[NST], s_empty[NST], s_full_u[32], s_full_v[8], s_acc_u[16], s_acc_v[8], s_vready[8];
+    __shared__ uint64_t s_acc_empty, s_acc_low, s_drain;
+    __shared__ uint32_t s_last[NST][2];           // loader: barrier (address) and 1 | parity << 8 of a stage's copies
     __shared__ uint32_t s_tmem;
     __shared__ volatile int s_err;
-    __shared__ float s_red[3][3][TP];             // partial sums of quarters 1..3: Re g, Im g, H
+    __shared__ float s_red[2][3][3][TP];          // by item parity: partial sums of quads 1..3: Re g, Im g, H
     const GeoDev& G = A.G;
-    const int n = G.n_elem, n2 = 2 * n;
-    // the elements e of U and V are taken in passes of ne (the accumulators of one pass
-    // fit TMEM); the contractions run over all r in every pass
-    const int ne = A.n_e, ne2 = 2 * ne;
-    const int npass = MULTI ? A.npass : 1;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    // U slices, then (when the Hessian diagonal is wanted) V slices
+    const AdjShape sh(G.n_elem);
+    const int n = sh.n;
+    const uint32_t ne = (uint32_t)sh.ne;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const bool want_h = A.want_h != 0;
-    const int nU = n2 / 16, nV = want_h ? n / 32 : 0, per = nU + nV;
+    const int n_ent = A.n_ent;
+    constexpr uint32_t kReads = 48;               // arrivals of the readers of a stage
     if (tid == 0) {
         for (int s = 0; s < NST; ++s) {
             tc::mbar_init(tc::smem_u32(&s_full[s]), 1);
-            tc::mbar_init(tc::smem_u32(&s_empty[s]), 1 + NPROD / 32);
+            tc::mbar_init(tc::smem_u32(&s_empty[s]), 1 + kReads);
         }
-        tc::mbar_init(tc::smem_u32(&s_acc_full), 1);
+        for (int d = 0; d < 32; ++d) tc::mbar_init(tc::smem_u32(&s_full_u[d]), 1);
+        for (int d = 0; d < 16; ++d) tc::mbar_init(tc::smem_u32(&s_acc_u[d]), 1);
+        for (int d = 0; d < 8; ++d) {
+            tc::mbar_init(tc::smem_u32(&s_full_v[d]), 1);
+            tc::mbar_init(tc::smem_u32(&s_acc_v[d]), 1);
+            tc::mbar_init(tc::smem_u32(&s_vready[d]), 8);
+        }
         tc::mbar_init(tc::smem_u32(&s_acc_empty), NPROD / 32);
         tc::mbar_init(tc::smem_u32(&s_acc_low), NPROD / 32);
-        tc::mbar_init(tc::smem_u32(&s_vready), NPROD / 32);
         tc::mbar_init(tc::smem_u32(&s_drain), 1);
         s_err = 0;
     }
@@ -272,717 +325,424 @@ __global__ void __launch_bounds__(NTHR_A, 1) k_adjoint_tc(TcArgs A) {
     tc::fence_before();
     __syncthreads();
     tc::fence_after();
-    const uint32_t tmem = s_tmem;
-    __nv_bfloat16* vimg = A.vimg + (size_t)blockIdx.x * (size_t)(n / 32) * (2 * TP * 32);
-    const int n_items = A.n_tiles * A.F.n;
-    const int my_items = (int)blockIdx.x < n_items ? (n_items - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
-    // slices of this CTA (a few thousand: 32-bit counters, stage and phase advanced
-    // incrementally, no divisions in the loops)
-    const int total = my_items * npass * per;
-    const size_t img_u = (size_t)n2 * 16, img_w = (size_t)n * 32;  // bf16 per hi (or lo) / W image slice
-    auto stage = [&](int s) { return smem + (size_t)s * ST_BYTES; };
+    const uint32_t tmem = __shfl_sync(0xffffffffu, s_tmem, 0);
+    const size_t vslice = 2 * TP * 32;            // bf16 of one |G|^2 slice (hi and lo)
+    __nv_bfloat16* vbuf = A.vimg + (size_t)blockIdx.x * 2 * (size_t)(n / 32) * vslice;
+    const int n_items = A.n_tiles * A.n_freq;
+    const uint32_t smem0 = tc::smem_u32(smem);
+    const uint32_t full0 = tc::smem_u32(&s_full[0]), full_u0 = tc::smem_u32(&s_full_u[0]), full_v0 = tc::smem_u32(&s_full_v[0]);
+    const uint32_t empty0 = tc::smem_u32(&s_empty[0]), acc_u0 = tc::smem_u32(&s_acc_u[0]), acc_v0 = tc::smem_u32(&s_acc_v[0]);
+    const uint32_t vready0 = tc::smem_u32(&s_vready[0]);
+    // full barrier of an entry, staged in s, and its parity (nd: parities of full[s])
+    auto full_bar = [&](AdjEnt e, uint32_t s) {
+        return e.diag() ? (e.is_v() ? full_v0 : full_u0) + 8u * e.d() : full0 + 8u * s;
+    };
 
     if (warp == NPROD / 32 + 1) {
         // ------------------------------ loader ------------------------------
-        if (lane == 0) {
-            int ql = 0, s = 0, j = 0, pass = 0, item = blockIdx.x;
-            int tile = item / A.F.n, fw = item - tile * A.F.n;
-            uint32_t ph = 0, vrp = 0;
-            bool err = false;
-            // the operand image streams through L2 once per launch: first out, so that it does
-            // not push the CTAs' G and |G|^2 scratch (rewritten every tile) out to DRAM
-            uint64_t stream_pol;
-            asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(stream_pol));
-            for (; ql < total; ++ql) {
-                // stage s = ql % NST with phase ph = (ql / NST) & 1; slice j of frequency fw of tile
-                if (ql >= NST && !tc::mbar_wait(tc::smem_u32(&s_empty[s]), ph ^ 1u, kMaxTries)) {
-                    err = true;
+        const bool lead = tc::elect_one();
+        int it = 0;
+        uint32_t ql = 0, s = 0, ph = 0, pass = 0, nd = 0;    // passes begun; bit s: parity of full[s]
+        bool ok = true;
+        // the operand image streams through L2 once per launch: first out, so that it does
+        // not push the CTAs' |G|^2 scratch (rewritten every tile) out to DRAM
+        uint64_t stream_pol;
+        asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(stream_pol));
+        for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x, ++it) {
+            const int tile = item / A.n_freq, fw = item - tile * A.n_freq;
+            const unsigned char* bu = A.bu + (size_t)fw * A.b_stride;
+            const unsigned char* bw = A.bw + (size_t)fw * A.b_stride;
+            const unsigned char* ap = (const unsigned char*)(A.aimg + (size_t)fw * A.aimg_stride +
+                                                             (size_t)tile * 2 * (n / 4) * 1024);
+            const unsigned char* const ap0 = ap;
+            const __nv_bfloat16* vimg = vbuf + (size_t)(it & 1) * (n / 32) * vslice;
+            for (int k = 0; k < n_ent; ++k, ++ql) {
+                const AdjEnt e = A.ent[k];
+                if (e.first()) {
+                    ++pass;
+                    ap = ap0;
+                }
+                if (ql >= NST && !tc::mbar_wait_warp(empty0 + 8u * s, ph ^ 1u, kMaxTries, &s_err)) {
+                    ok = false;
                     break;
                 }
-                if (s_err) break;
-                const uint32_t mb = tc::smem_u32(&s_full[s]);
-                if (j < nU) {
-                    const uint32_t abytes = TP * 16 * 2, bbytes = (uint32_t)(ne2 * 64);
-                    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(mb), "r"(2u * abytes + bbytes)
-                                 : "memory");
-                    // image rows 2j, 2j + 1 of the hi plane, then of the lo plane
-                    const __nv_bfloat16* asrc =
-                        A.aimg + (size_t)fw * A.aimg_stride + ((size_t)tile * 2 * (n2 / 8) + 2 * j) * 1024;
-                    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint"
-                                 " [%0], [%1], %2, [%3], %4;"
-                                 ::"r"(tc::smem_u32(stage(s))), "l"(asrc), "r"(abytes), "r"(mb), "l"(stream_pol)
-                                 : "memory");
-                    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint"
-                                 " [%0], [%1], %2, [%3], %4;"
-                                 ::"r"(tc::smem_u32(stage(s) + ST_ALO)), "l"(asrc + (size_t)(n2 / 8) * 1024), "r"(abytes),
-                                 "r"(mb), "l"(stream_pol)
-                                 : "memory");
-                    // B: rows e' of this pass (contiguous in each plane), hi then lo; with one
-                    // pass the two planes are adjacent and go in one copy
-                    const __nv_bfloat16* bsrc = A.bu + (size_t)fw * A.bu_stride + (size_t)j * 2 * img_u + (size_t)pass * ne2 * 16;
-                    if (!MULTI) {
-                        asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                                     ::"r"(tc::smem_u32(stage(s) + ST_B)), "l"(bsrc), "r"(bbytes), "r"(mb)
-                                     : "memory");
-                    } else {
-                        asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                                     ::"r"(tc::smem_u32(stage(s) + ST_B)), "l"(bsrc), "r"(bbytes / 2), "r"(mb)
-                                     : "memory");
-                        asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                                     ::"r"(tc::smem_u32(stage(s) + ST_B + bbytes / 2)), "l"(bsrc + img_u), "r"(bbytes / 2),
-                                     "r"(mb)
-                                     : "memory");
+                uint32_t dst = smem0 + s * ST_BYTES;
+                const uint32_t par = e.diag() ? (pass - 1u) & 1u : (nd >> s) & 1u;
+                const uint32_t mb = full_bar(e, s);
+                if (!e.diag()) nd ^= 1u << s;
+                if (e.is_v() && e.diag() && !tc::mbar_wait_warp(vready0 + 8u * e.d(), par, kMaxTries, &s_err)) {
+                    // the |G|^2 slice, written by the quads (a slice below the diagonal in an earlier
+                    // pass of the item), did not come: nothing issued into this stage
+                    ok = false;
+                    break;
+                }
+                if (!e.is_v()) {
+                    // rows of the entry's slices: 2 ne below the diagonal (cnt = 1), then 16 fewer each
+                    const uint32_t cnt = e.cnt();
+                    uint32_t bb = 64u * (2u * ne - 16u * e.d());
+                    if (lead) tc::bulk_arm(mb, cnt * (ST_B + bb) - 512u * cnt * (cnt - 1u));
+                    for (uint32_t c = 0; c < cnt; ++c) {
+                        if (lead) {
+                            // image rows 2j, 2j + 1 of the hi plane, then of the lo plane
+                            tc::bulk_copy(dst + ST_B, bu, bb, mb);
+                            tc::bulk_copy_hint(dst, ap, 4096u, mb, stream_pol);
+                            tc::bulk_copy_hint(dst + ST_ALO, ap + (size_t)(n / 4) * 2048, 4096u, mb, stream_pol);
+                        }
+                        ap += 4096;
+                        bu += bb;
+                        dst += ST_B + bb;
+                        bb -= 1024u;
                     }
                 } else {
-                    if (j == nU) {
-                        // this (tile, frequency)'s |G|^2 slices are written by the producers
-                        if (!tc::mbar_wait(tc::smem_u32(&s_vready), vrp & 1u, kMaxTries)) {
-                            err = true;
-                            break;
-                        }
-                        ++vrp;
+                    const uint32_t wbytes = 64u * (ne - 32u * e.d()), abytes = 2u * TP * 32 * 2;
+                    if (lead) {
+                        tc::bulk_arm(mb, wbytes + abytes);
+                        tc::bulk_copy(dst + ST_VB, bw, wbytes, mb);
+                        tc::bulk_copy(dst, vimg + (size_t)e.j() * vslice, abytes, mb);
                     }
-                    const uint32_t wbytes = (uint32_t)(ne * 64), abytes = 2u * TP * 32 * 2;
-                    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(mb), "r"(wbytes + abytes)
-                                 : "memory");
-                    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                                 ::"r"(tc::smem_u32(stage(s) + ST_VB)),
-                                 "l"(A.bw + (size_t)fw * A.bw_stride + (size_t)(j - nU) * img_w + (size_t)pass * ne * 32),
-                                 "r"(wbytes), "r"(mb)
-                                 : "memory");
-                    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                                 ::"r"(tc::smem_u32(stage(s))), "l"(vimg + (size_t)(j - nU) * (2 * TP * 32)), "r"(abytes),
-                                 "r"(mb)
-                                 : "memory");
+                    bw += wbytes;
+                }
+                if (lead) {
+                    s_last[s][0] = mb;
+                    s_last[s][1] = par;
                 }
                 if (++s == NST) { s = 0; ph ^= 1u; }
-                if (++j == per) {
-                    j = 0;
-                    if (++pass == npass) {
-                        pass = 0;
-                        item += gridDim.x;
-                        tile = item / A.F.n;
-                        fw = item - tile * A.F.n;
-                    }
-                }
             }
-            if (err || s_err) {
-                s_err = 1;
-                // bounded waits for the last copies issued (at most one per stage)
-                for (int x = (ql > NST ? ql - NST : 0); x < ql; ++x)
-                    tc::mbar_wait(tc::smem_u32(&s_full[x % NST]), (uint32_t)(x / NST) & 1u, kMaxTries);
-            }
+        }
+        if (!ok && lead) {
+            s_err = 1;
+            // bounded waits for the last copies issued into each stage
+            for (uint32_t x = 0; x < (ql < NST ? ql : (uint32_t)NST); ++x) tc::mbar_wait(s_last[x][0], s_last[x][1], kMaxTries);
         }
         __syncwarp();
     } else if (warp == NPROD / 32) {
         // ------------------------------ MMA issuer ------------------------------
-        if (lane == 0) {
-            const int nbk = ne2 > 256 ? 2 : 1;
-            const int nb_u = ne2 / nbk;
-            const uint32_t id_u = tc::idesc_bf16_f32(128, (uint32_t)nb_u);
-            const uint32_t id_v = tc::idesc_bf16_f32(128, (uint32_t)ne);
-            int s = 0, j = 0;
-            uint32_t acce = 0, accl = 0, ph = 0;
-            bool err = false, issued = false;
-            for (int q = 0; q < total && !err; ++q) {
-                if (j == nU) {
-                    // V overwrites the columns of the first N-block of U: its part of the U
-                    // epilogue must be done (the rest of it overlaps the V MMAs)
-                    if (!tc::mbar_wait(tc::smem_u32(&s_acc_low), accl & 1u, kMaxTries)) { err = true; break; }
-                    ++accl;
-                } else if (j == 0 && q > 0) {
-                    // a new U phase: the V epilogue must have read the accumulator
-                    if (!tc::mbar_wait(tc::smem_u32(&s_acc_empty), acce & 1u, kMaxTries)) { err = true; break; }
-                    ++acce;
+        const bool lead = tc::elect_one();
+        const uint32_t id0 = tc::idesc_bf16_f32(128, 0);
+        uint32_t s = 0, pass = 0, nd = 0;
+        bool ok = true, begun = false;
+        AdjEnt e = A.ent[0];
+        for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
+            bool v_begun = false;
+            for (int k = 0; k < n_ent; ++k) {
+                const AdjEnt nx = A.ent[k + 1 < n_ent ? k + 1 : 0];   // in time for the next round
+                if (e.first()) {
+                    // a new pass: every column of the previous one must have been read
+                    if (pass > 0) ok = tc::mbar_wait_warp(tc::smem_u32(&s_acc_empty), (pass - 1u) & 1u, kMaxTries, &s_err);
+                    ++pass;
+                    v_begun = false;
                 }
-                if (!tc::mbar_wait(tc::smem_u32(&s_full[s]), ph, kMaxTries)) { err = true; break; }
-                if (s_err) { err = true; break; }
+                if (e.is_v() && !v_begun) {
+                    if (A.low_groups > 0) ok = ok && tc::mbar_wait_warp(tc::smem_u32(&s_acc_low), (pass - 1u) & 1u, kMaxTries, &s_err);
+                    v_begun = true;
+                }
+                if (!ok) break;
+                ok = tc::mbar_wait_warp(full_bar(e, s), e.diag() ? (pass - 1u) & 1u : (nd >> s) & 1u, kMaxTries, &s_err);
+                if (!ok) break;
                 tc::fence_after();
-                const uint32_t sa = tc::smem_u32(stage(s)), sal = sa + ST_ALO, sb = sa + ST_B;
-                // U: A K-major in the image's arrangement: K cores 2048 B apart (LBO), 8-pixel
-                // cores 128 B apart (SBO)
-                const uint64_t dah = tc::sdesc(sa, 2048, 128), dal = tc::sdesc(sal, 2048, 128);
-                if (j < nU) {
-                    const uint32_t acc = j > 0 ? 1u : 0u;
-                    for (int nb = 0; nb < nbk; ++nb) {
-                        const uint32_t boff = (uint32_t)(nb * nb_u / 8) * 256u;
-                        const uint64_t dbh = tc::sdesc(sb + boff, 128, 256);
-                        const uint64_t dbl = tc::sdesc(sb + (uint32_t)(ne2 * 32) + boff, 128, 256);
-                        const uint32_t d = tmem + (uint32_t)(nb * nb_u);
-                        tc::mma_bf16(d, dah, dbh, id_u, acc);
-                        tc::mma_bf16(d, dah, dbl, id_u, 1u);
-                        tc::mma_bf16(d, dal, dbh, id_u, 1u);
+                const uint32_t sa0 = smem0 + s * ST_BYTES;
+                if (!e.is_v()) {
+                    uint32_t sa = sa0, rows = 2u * ne - 16u * e.d(), col = tmem + 16u * e.d();
+                    uint32_t acc = e.j() > 0u ? 1u : 0u;
+                    const uint32_t cnt = e.cnt();
+                    for (uint32_t c = 0; c < cnt; ++c) {
+                        // A K-major in the image's arrangement: K cores 2048 B apart (LBO), 8-pixel
+                        // cores 128 B apart (SBO)
+                        const uint64_t dah = tc::sdesc(sa, 2048, 128), dal = tc::sdesc(sa + ST_ALO, 2048, 128);
+                        const uint64_t dbh = tc::sdesc(sa + ST_B, 128, 256), dbl = tc::sdesc(sa + ST_B + 32u * rows, 128, 256);
+                        // one or two N-blocks: what exceeds 256 columns, then the last 256 (a row of B is 32 bytes)
+                        const uint32_t n1 = rows > 256u ? rows - 256u : rows, id1 = id0 | ((n1 >> 3) << 17);
+                        if (lead) {
+                            tc::mma_bf16(col, dah, dbh, id1, acc);
+                            tc::mma_bf16(col, dah, dbl, id1, 1u);
+                            tc::mma_bf16(col, dal, dbh, id1, 1u);
+                            if (rows > 256u) {
+                                const uint32_t id2 = id0 | ((256u >> 3) << 17), c2 = col + n1;
+                                const uint64_t dbh2 = dbh + 2u * n1, dbl2 = dbl + 2u * n1;
+                                tc::mma_bf16(c2, dah, dbh2, id2, acc);
+                                tc::mma_bf16(c2, dah, dbl2, id2, 1u);
+                                tc::mma_bf16(c2, dal, dbh2, id2, 1u);
+                            }
+                            if (e.diag() && ((e.d() + c) & 1u)) tc::commit(acc_u0 + 8u * ((e.d() + c) >> 1));
+                        }
+                        sa += ST_B + 64u * rows;
+                        col += 16u;
+                        rows -= 16u;
+                        acc = 1u;
                     }
                 } else {
-                    // K = 32 slice in the chunk_offset layout (SBO = 512): two K = 16 steps
-#pragma unroll
-                    for (int kh = 0; kh < 2; ++kh) {
-                        const uint64_t vah = tc::sdesc(sa + 256u * kh, 128, 512);
-                        const uint64_t val = tc::sdesc(sa + ST_VALO + 256u * kh, 128, 512);
-                        const uint64_t vb = tc::sdesc(sa + ST_VB + 256u * kh, 128, 512);
-                        tc::mma_bf16(tmem, vah, vb, id_v, (j > nU || kh > 0) ? 1u : 0u);
-                        tc::mma_bf16(tmem, val, vb, id_v, 1u);
+                    const uint32_t rows = ne - 32u * e.d(), id = id0 | ((rows >> 3) << 17);
+                    const uint32_t d = tmem + A.v_col + 32u * e.d();
+                    // K = 32 slice in the chunk_offset layout (SBO = 512): two K = 16 steps, 256 bytes apart
+                    const uint64_t vah = tc::sdesc(sa0, 128, 512), val = tc::sdesc(sa0 + ST_VALO, 128, 512);
+                    const uint64_t vb = tc::sdesc(sa0 + ST_VB, 128, 512);
+                    if (lead) {
+                        tc::mma_bf16(d, vah, vb, id, e.j() > 0u ? 1u : 0u);
+                        tc::mma_bf16(d, val, vb, id, 1u);
+                        tc::mma_bf16(d, vah + 16u, vb + 16u, id, 1u);
+                        tc::mma_bf16(d, val + 16u, vb + 16u, id, 1u);
+                        if (e.diag()) tc::commit(acc_v0 + 8u * e.d());
                     }
                 }
-                issued = true;
-                tc::commit(tc::smem_u32(&s_empty[s]));
-                if (j == nU - 1 || j == per - 1) tc::commit(tc::smem_u32(&s_acc_full));
-                if (++s == NST) { s = 0; ph ^= 1u; }
-                if (++j == per) j = 0;
-            }
-            if (err) {
-                s_err = 1;
-                atomicAdd(A.counters + CNT_TC_TIMEOUT, 1u);
-                // bounded wait for the MMAs still in flight
-                if (issued) {
-                    tc::commit(tc::smem_u32(&s_drain));
-                    tc::mbar_wait(tc::smem_u32(&s_drain), 0u, kMaxTries);
+                begun = true;
+                if (lead) {
+                    tc::commit(empty0 + 8u * s);
+                    if (!e.diag()) tc::mbar_arrive_cnt(empty0 + 8u * s, kReads);
                 }
+                if (!e.diag()) nd ^= 1u << s;
+                if (++s == NST) s = 0;
+                e = nx;
+            }
+        }
+        if (!ok && lead) {
+            s_err = 1;
+            atomicAdd(A.counters + CNT_TC_TIMEOUT, 1u);
+            // bounded wait for the MMAs still in flight
+            if (begun) {
+                tc::commit(tc::smem_u32(&s_drain));
+                tc::mbar_wait(tc::smem_u32(&s_drain), 0u, kMaxTries);
             }
         }
         __syncwarp();
     } else {
-        // -------------------------------- producers --------------------------------
-        const uint32_t p = (uint32_t)(tid & (TP - 1)), h = (uint32_t)(tid / TP);
-        const uint32_t lane_off = (uint32_t)((warp & 3) * 32) << 16;
-        // the U slices' (pixel, quarter) items go 8 pixels x 4 quarters to a warp: the A reads
-        // then fall on distinct shared-memory banks and the |G|^2 stores on 128 contiguous
-        // bytes (the epilogues keep p = the TMEM lane)
-        const uint32_t cp = (uint32_t)((lane & 7) + 8 * warp), ch = (uint32_t)(lane >> 3);
-        float2* gs = A.gscr + (size_t)blockIdx.x * n * TP;
-        bool err = false;
-        int qs = 0;                // stage of the next slice
-        uint32_t qph = 0;          // its phase
-        uint32_t accf = 0;
-        // one slice: wait for its stage to be filled, use it, release it
-        auto slice = [&](auto&& consume) {
-            const int s = qs;
-            if (!err) err = !tc::mbar_wait(tc::smem_u32(&s_full[s]), qph, kMaxTries);
-            err = __any_sync(0xffffffffu, err || s_err != 0);
-            if (!err) consume(stage(s), stage(s) + ST_ALO);
+        // ------------------------------ epilogue quads ------------------------------
+        const uint32_t p = (uint32_t)(tid & (TP - 1));
+        const int quad = warp >> 2;
+        const uint32_t t0 = tmem + ((uint32_t)((warp & 3) * 32) << 16);
+        const unsigned char* const a_base = smem + (p >> 3) * 128u + (p & 7u) * 16u;   // this pixel in a K core of an A slice
+        const int n_work = A.n_work[quad];
+        bool ok = true;
+        int it = 0;
+        uint32_t s0 = 0, pass = 0;    // stage of the item's first entry
+        auto wait = [&](uint32_t bar, uint32_t parity) {
+            if (ok) ok = tc::mbar_wait_warp(bar, parity, kMaxTries, &s_err);
+            return ok;
+        };
+        auto arrive = [&](uint32_t bar, uint32_t cnt) {
             __syncwarp();
-            if (lane == 0 && !err) tc::mbar_arrive(tc::smem_u32(&s_empty[s]));
-            if (++qs == NST) { qs = 0; qph ^= 1u; }
+            if (lane == 0) tc::mbar_arrive_cnt(bar, cnt);
         };
-        // wait for the accumulator of the phase just issued (warp-uniform result)
-        auto acc_wait = [&]() {
-            if (!err) err = !tc::mbar_wait(tc::smem_u32(&s_acc_full), accf & 1u, kMaxTries);
-            ++accf;
-            err = __any_sync(0xffffffffu, err);
-            tc::fence_after();
+        auto stage_of = [&](uint32_t f) {   // of a work record's a or b
+            const uint32_t s = s0 + (f & 15u);
+            return s >= (uint32_t)NST ? s - NST : s;
         };
-        auto acc_release = [&]() {
-            tc::fence_before();
-            __syncwarp();
-            if (lane == 0 && !err) tc::mbar_arrive(tc::smem_u32(&s_acc_empty));
-        };
-        // items (tile, frequency), item = tile F.n + fw, dealt to the CTAs in turn
-        for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
-            const int tile = item / A.F.n, fw = item - (item / A.F.n) * A.F.n;
-            const int px = tile * TP + (int)p;
-            const bool valid = px < G.npix;
-            {
-                const FreqC fc = A.F.f[fw];
-                float fg_r = 0.f, fg_i = 0.f, fh = 0.f;   // this frequency's g and H, summed over the passes
-                for (int pass = 0; pass < npass; ++pass) {
-                const int eb0 = pass * ne;                 // first element of this pass
-                // ---- U slices: exact-enough G for the epilogue and the |G|^2 slices ----
-                for (int j = 0; j < nU; ++j)
-                    slice([&](const unsigned char* ahi, const unsigned char* alo) {
-                        consume_u(j * 8, cp, ch, ahi, alo, gs, vimg, want_h);
-                    });
-                // the |G|^2 slices (read next by the bulk copies of the loader) are complete
-                if (want_h) {
-                    asm volatile("fence.proxy.async.global;" ::: "memory");
-                    __syncwarp();
-                    if (lane == 0 && !err) tc::mbar_arrive(tc::smem_u32(&s_vready));
-                }
-                // gs (G of the tile) is complete
-                err = tc::named_or(1, NPROD, err);
-                if (err) break;
-                // ---- U epilogue: element chunks of 8, e0 = 32 b + 8 c for blocks b = h, h + 4, ...
-                // and c < 4 (in increasing e); element e's Re U is in column nbu (e / ebu) + e % ebu
-                // and its Im U ebu columns further (N-blocks of nbu columns, ebu = nbu / 2
-                // elements each); G of the next chunk is loaded while the current one is used,
-                // the first before the accumulator wait ----
-                const int nch = 4 * ((ne / 32 - (int)h + 3) / 4);
-                const int nbu = ne2 > 256 ? ne2 / 2 : ne2, ebu = nbu / 2;
-                auto ce0 = [&](int k) { return 32 * ((int)h + 4 * (k >> 2)) + 8 * (k & 3); };
-                auto recol = [&](int e) { return (e / ebu) * nbu + e % ebu; };
-                auto gload = [&](int k, float2 (&g)[8]) {
-                    const int e0 = ce0(k);
+        for (int item = blockIdx.x; item < n_items; item += gridDim.x, ++it) {
+            const int tile = item / A.n_freq, fw = item - tile * A.n_freq;
+            __nv_bfloat16* vimg = vbuf + (size_t)(it & 1) * (n / 32) * vslice;
+            float gr = 0.f, gi = 0.f, hh = 0.f;
+            for (int k = 0; k < n_work && ok; ++k) {
+                const AdjWork w = A.work[quad][k];
+                if (w.first()) ++pass;
+                const uint32_t par = (pass - 1u) & 1u, u = w.u();
+                const uint32_t sa = stage_of(w.a);
+                if (!w.is_v()) {
+                    // G of the unit's 16 elements: K core h of a slice holds elements 4 h .. 4 h + 3
+                    // as (Re G, -Im G) pairs, in a hi and a lo plane
+                    uint4 hv[4], lv[4];
+                    if (!wait(full_u0 + 8u * (w.a >> 16), par)) break;
+                    const unsigned char* ap = a_base + sa * ST_BYTES + ((w.a >> 4) & 0xffu) * 1024u;
+                    hv[0] = *(const uint4*)ap;
+                    hv[1] = *(const uint4*)(ap + 2048);
+                    lv[0] = *(const uint4*)(ap + ST_ALO);
+                    lv[1] = *(const uint4*)(ap + ST_ALO + 2048);
+                    uint32_t sb = sa;
+                    if (w.b != 0u) {
+                        arrive(empty0 + 8u * sa, (w.a >> 12) & 15u);
+                        if (!wait(full_u0 + 8u * (w.b >> 16), par)) break;
+                        sb = stage_of(w.b);
+                        ap = a_base + sb * ST_BYTES + ((w.b >> 4) & 0xffu) * 1024u;
+                    } else {
+                        ap = a_base + sa * ST_BYTES + w.off2 * 1024u;
+                    }
+                    hv[2] = *(const uint4*)ap;
+                    hv[3] = *(const uint4*)(ap + 2048);
+                    lv[2] = *(const uint4*)(ap + ST_ALO);
+                    lv[3] = *(const uint4*)(ap + ST_ALO + 2048);
+                    arrive(empty0 + 8u * sb, ((w.b != 0u ? w.b : w.a) >> 12) & 15u);
+                    float x[16], y[16];   // Re G, -Im G
 #pragma unroll
-                    for (int i = 0; i < 8; ++i) g[i] = gs[(size_t)(eb0 + e0 + i) * TP + p];
-                };
-                auto gchunk = [&](int k, const float2 (&g)[8], float& ar, float& ai) {
-                    const int e0 = ce0(k);
-                    float vr[8], vi[8];
-                    tc::tmem_ld8(tmem + lane_off + (uint32_t)recol(e0), vr);
-                    tc::tmem_ld8(tmem + lane_off + (uint32_t)(recol(e0) + ebu), vi);
+                    for (int i = 0; i < 4; ++i) {
+                        const uint32_t hw[4] = {hv[i].x, hv[i].y, hv[i].z, hv[i].w}, lw[4] = {lv[i].x, lv[i].y, lv[i].z, lv[i].w};
 #pragma unroll
-                    for (int i = 0; i < 8; ++i) {
-                        ar = fmaf(g[i].x, vr[i], fmaf(g[i].y, vi[i], ar));
-                        ai = fmaf(g[i].x, vi[i], fmaf(-g[i].y, vr[i], ai));
+                        for (int e = 0; e < 4; ++e) {
+                            x[4 * i + e] = sum_lo16(hw[e], lw[e]);
+                            y[4 * i + e] = sum_hi16(hw[e], lw[e]);
+                        }
                     }
-                };
-                // the V MMAs write columns [0, n), inside the first N-block: released once this
-                // warp has read its chunks of elements < ebu
-                bool low = false;
-                auto release_low = [&]() {
-                    tc::fence_before();
-                    __syncwarp();
-                    if (lane == 0 && !err) tc::mbar_arrive(tc::smem_u32(&s_acc_low));
-                    low = true;
-                };
-                float2 ga[8], gb[8];
-                if (nch > 0) gload(0, ga);
-                acc_wait();
-                float gr = 0.f, gi = 0.f;
-                if (!err) {
-                    for (int k = 0; k < nch; k += 2) {
-                        if (!low && ce0(k) >= ebu) release_low();
-                        gload(k + 1, gb);
-                        gchunk(k, ga, gr, gi);
-                        if (k + 2 < nch) gload(k + 2, ga);
-                        gchunk(k + 1, gb, gr, gi);
+                    if (want_h) {
+                        // elements 16 u .. 16 u + 15 of the pass: cores 2 (u % 2), + 1 of its V slice u / 2
+                        __nv_bfloat16* vs = vimg + (size_t)(w.q() * (uint32_t)sh.gv + (u >> 1)) * vslice +
+                                            tc::chunk_offset(p, 16u * (u & 1u)) / 2;
+#pragma unroll
+                        for (int c = 0; c < 2; ++c) {
+                            uint32_t vh[4], vl[4];
+#pragma unroll
+                            for (int i = 0; i < 4; ++i) {
+                                __nv_bfloat16 a, b, al, bl;
+                                const int e0 = 8 * c + 2 * i, e1 = e0 + 1;
+                                tc::split_bf16(x[e0] * x[e0] + y[e0] * y[e0], a, al);
+                                tc::split_bf16(x[e1] * x[e1] + y[e1] * y[e1], b, bl);
+                                vh[i] = pack2(a, b);
+                                vl[i] = pack2(al, bl);
+                            }
+                            *(uint4*)(vs + 64 * c) = make_uint4(vh[0], vh[1], vh[2], vh[3]);
+                            *(uint4*)(vs + 64 * c + TP * 32) = make_uint4(vl[0], vl[1], vl[2], vl[3]);
+                        }
+                        asm volatile("fence.proxy.async.global;" ::: "memory");   // read next by the loader's bulk copies
+                        arrive(vready0 + 8u * (u >> 1), 1u);
                     }
-                }
-                if (!low) release_low();
-                if (h > 0) {
-                    s_red[0][h - 1][p] = gr;
-                    s_red[1][h - 1][p] = gi;
-                }
-                err = tc::named_or(1, NPROD, err);
-                if (err) break;
-                if (h == 0) {
-                    fg_r += (gr + s_red[0][0][p] + s_red[0][1][p] + s_red[0][2][p]) * fc.w2;
-                    fg_i += (gi + s_red[1][0][p] + s_red[1][1][p] + s_red[1][2][p]) * fc.w2;
-                }
-                if (!want_h) {
-                    // no V phase: the accumulator is free for the next U phase
-                    acc_release();
-                    continue;
-                }
-                // ---- V slices: A and B come by bulk copy; the producers only pass the
-                // stage barriers, which keeps every stage's phases in step with its uses ----
-                for (int j = 0; j < nV; ++j) slice([&](const unsigned char*, const unsigned char*) {});
-                // ---- V epilogue (same chunks, |G|^2 against V in columns e) ----
-                uint4 qa[2], qb[2];
-                if (nch > 0) g2_load(vimg, eb0 + ce0(0), p, qa);
-                acc_wait();
-                float hh = 0.f;
-                if (!err) {
-                    for (int k = 0; k < nch; k += 2) {
-                        g2_load(vimg, eb0 + ce0(k + 1), p, qb);
-                        h_chunk(tmem + lane_off + (uint32_t)ce0(k), qa, hh);
-                        if (k + 2 < nch) g2_load(vimg, eb0 + ce0(k + 2), p, qa);
-                        h_chunk(tmem + lane_off + (uint32_t)ce0(k + 1), qb, hh);
+                    if (!wait(acc_u0 + 8u * u, par)) break;
+                    tc::fence_after();
+                    float v[32];   // per group of 8 elements: Re U, then Im U
+                    tc::tmem_ld32(t0 + 32u * u, v);
+                    // the columns V takes over (or the next pass) are free once read
+                    if (w.low() || w.last()) tc::fence_before();
+                    if (w.low()) arrive(tc::smem_u32(&s_acc_low), 1u);
+                    if (w.last()) arrive(tc::smem_u32(&s_acc_empty), 1u);
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) {
+                        const float ur = v[16 * (i >> 3) + (i & 7)], ui = v[16 * (i >> 3) + 8 + (i & 7)];
+                        gr = fmaf(x[i], ur, fmaf(-y[i], ui, gr));
+                        gi = fmaf(x[i], ui, fmaf(y[i], ur, gi));
                     }
-                }
-                acc_release();
-                if (h > 0) s_red[2][h - 1][p] = hh;
-                err = tc::named_or(1, NPROD, err);
-                if (err) break;
-                if (h == 0) fh += (hh + s_red[2][0][p] + s_red[2][1][p] + s_red[2][2][p]) * fc.w4;
-                }   // passes
-                if (err) break;
-                if (h == 0 && valid) {
-                    if (A.g_out) A.g_out[(size_t)fw * G.npix + px] = make_float2(fg_r, fg_i);
-                    if (A.h_out) A.h_out[(size_t)fw * G.npix + px] = fh;
-                    // this frequency's Re g and H for the sums over the set (k_adjoint_sums)
-                    if (A.fpart) A.fpart[(size_t)fw * G.npix + px] = make_float2(fg_r, fh);
+                } else {
+                    if (!wait(full_v0 + 8u * u, par)) break;
+                    const unsigned char* ap = smem + sa * ST_BYTES + (p >> 3) * 512u + (p & 7u) * 16u;
+                    uint4 h[4], l[4];   // |G|^2 of elements 8 x .. 8 x + 7, hi and lo planes
+#pragma unroll
+                    for (int x = 0; x < 4; ++x) {
+                        h[x] = *(const uint4*)(ap + 128 * x);
+                        l[x] = *(const uint4*)(ap + ST_VALO + 128 * x);
+                    }
+                    arrive(empty0 + 8u * sa, kReads / 4u);
+                    if (!wait(acc_v0 + 8u * u, par)) break;
+                    tc::fence_after();
+                    float v[32];
+                    tc::tmem_ld32(t0 + A.v_col + 32u * u, v);
+                    if (w.last()) {
+                        tc::fence_before();
+                        arrive(tc::smem_u32(&s_acc_empty), 1u);
+                    }
+#pragma unroll
+                    for (int x = 0; x < 4; ++x) {
+                        const uint32_t hw[4] = {h[x].x, h[x].y, h[x].z, h[x].w}, lw[4] = {l[x].x, l[x].y, l[x].z, l[x].w};
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            hh = fmaf(sum_lo16(hw[i], lw[i]), v[8 * x + 2 * i], hh);
+                            hh = fmaf(sum_hi16(hw[i], lw[i]), v[8 * x + 2 * i + 1], hh);
+                        }
+                    }
                 }
             }
-            if (err) break;
+            s0 = (s0 + (uint32_t)n_ent) % NST;
+            // the quads' sums, in fixed order
+            float(*red)[3][TP] = s_red[it & 1];
+            if (quad > 0) {
+                red[quad - 1][0][p] = gr;
+                red[quad - 1][1][p] = gi;
+                red[quad - 1][2][p] = hh;
+            }
+            if (tc::named_or(1, NPROD, !ok)) {
+                ok = false;
+                break;
+            }
+            const int px = tile * TP + (int)p;
+            if (quad == 0 && px < G.npix) {
+                const float fr = (gr + red[0][0][p] + red[1][0][p] + red[2][0][p]) * A.w2[fw];
+                const float fi = (gi + red[0][1][p] + red[1][1][p] + red[2][1][p]) * A.w2[fw];
+                const float fh = (hh + red[0][2][p] + red[1][2][p] + red[2][2][p]) * A.w4[fw];
+                const size_t o = (size_t)fw * G.npix + px;
+                if (A.g_out) A.g_out[o] = make_float2(fr, fi);
+                if (A.h_out) A.h_out[o] = fh;
+                // this frequency's Re g and H for the sums over the set (k_adjoint_sums)
+                if (A.fpart) A.fpart[o] = make_float2(fr, fh);
+            }
         }
+        if (!ok) s_err = 1;
     }
     tc::fence_before();
     __syncthreads();
     if (warp == 0) tc::tmem_dealloc(tmem, A.tmem_cols);
 }
-// ---------------------------------------------------------------------------
-// The same adjoint on CTA pairs (a cluster of two CTAs, cta_group::2 MMAs of M = 256).
-// The pair takes two 128-pixel tiles at a time, one per CTA (a pair with one tile left
-// takes the last tile twice and keeps one result), and each CTA stages only its own
-// half of every operand: its tile's A slices and half the rows of each N-block of S
-// (and of W).  The MMA over both CTAs' shared memory then reads half the S bytes per
-// CTA that the single-CTA kernel reads, and the stages (A 8 KB + S half 16 KB) are
-// 24 KB instead of 40, so eight of them fit.  Each CTA's TMEM holds its own tile's U
-// and V (128 lanes), so the producers and epilogues are those of the single-CTA
-// kernel.  Roles as there, plus:
-//   rank 0, warp 16: MMA issuer for the pair: waits for its own stage and for the
-//               peer's ("pfull", arrived on from the peer), issues the pair MMAs and
-//               commits them to the "empty" (and accumulator) barriers of both CTAs;
-//   rank 1, warp 16: relay: when a stage of its CTA is filled, arrives on the
-//               issuer's pfull for it;
-//   the accumulator barriers the issuer waits for (acc_empty, acc_low) take the
-//   arrivals of both CTAs' producer warps.
-// Every wait is bounded; both CTAs meet at a cluster barrier before they free TMEM
-// and exit, so no CTA leaves while its peer may still touch its shared memory.
-// ---------------------------------------------------------------------------
-constexpr int NST2 = 8;
-constexpr uint32_t ST2_BYTES = 24u * 1024u;
-// U stage: A hi (4 KB), A lo (4 KB), then this CTA's S rows of every N-block (hi for each
-// N-block, then lo); V stage: |G|^2 hi (8 KB), lo (8 KB), this CTA's W rows (<= 8 KB)
-constexpr uint32_t ST2_ALO = 4096u, ST2_B = 8192u, ST2_VALO = 8192u, ST2_VB = 16384u;
 
-template <bool MULTI>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHR_A, 1) k_adjoint_tc2(TcArgs A) {
-    extern __shared__ __align__(1024) unsigned char smem[];
-    __shared__ uint64_t s_full[NST2], s_pfull[NST2], s_empty[NST2], s_acc_full, s_acc_empty, s_acc_low, s_vready, s_drain;
-    __shared__ uint32_t s_tmem;
-    __shared__ volatile int s_err;
-    __shared__ float s_red[3][3][TP];             // partial sums of quarters 1..3: Re g, Im g, H
-    const GeoDev& G = A.G;
-    const int n = G.n_elem, n2 = 2 * n;
-    const int ne = A.n_e, ne2 = 2 * ne;
-    const int npass = MULTI ? A.npass : 1;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const uint32_t rank = tc::cluster_ctarank();   // 0 issues the pair's MMAs
-    const bool want_h = A.want_h != 0;
-    const int nU = n2 / 16, nV = want_h ? n / 32 : 0, per = nU + nV;
-    // N-blocks of U (as in the single-CTA kernel) and this CTA's half of each
-    const int nbk = ne2 > 256 ? 2 : 1, nb_u = ne2 / nbk, hrow = nb_u / 2;
-    const uint32_t hb = (uint32_t)hrow * 32u;    // bytes of one plane of one N-block half
-    const int wrow = ne / 2;                     // this CTA's W rows
-    if (tid == 0) {
-        for (int s = 0; s < NST2; ++s) {
-            tc::mbar_init(tc::smem_u32(&s_full[s]), 1);
-            tc::mbar_init(tc::smem_u32(&s_pfull[s]), 1);
-            tc::mbar_init(tc::smem_u32(&s_empty[s]), 1 + NPROD / 32);
+// The slices of one (tile, frequency) in order, one entry per pipeline stage, and each
+// quad's work records in the same order: per pass the U slices with r ascending (the short
+// diagonal ones packed up to four to a 40 KB stage), and each V slice ADJ_V_LAG U stages
+// behind the last U group it depends on: the group whose |G|^2 it reads (its bulk copy
+// would otherwise wait for a slice just landed) and, where V takes over U columns, the last
+// of those.  False if the tables are too small (no supported ring size).
+constexpr int ADJ_V_LAG = 3;
+bool adj_schedule(const AdjShape& sh, bool want_h, int low_groups, TcArgs* A) {
+    int k = 0;
+    bool fits = true;
+    for (int i = 0; i < 4; ++i) A->n_work[i] = 0;
+    for (int q = 0; q < sh.n / sh.ne; ++q) {
+        const int nu = (q + 1) * sh.ge, nv = want_h ? (q + 1) * sh.gv : 0, dj = q * sh.ge, dv = q * sh.gv;
+        int stage_of[32];              // U stage (in this pass) of each diagonal group
+        uint32_t where[32], off[32];   // its record field a / b, and its KB offset in the stage
+        bool begun[4] = {false, false, false, false};
+        auto put = [&](int j, int cnt, bool v, bool first, int d) {
+            if (k < ADJ_MAX_ENT) A->ent[k] = AdjEnt::make(j, cnt, v, first, d);
+            else fits = false;
+            ++k;
+        };
+        auto work = [&](int quad, uint32_t x, uint32_t a, uint32_t b, uint32_t off2) {
+            int& m = A->n_work[quad];
+            if (m < ADJ_MAX_WORK)
+                A->work[quad][m] = AdjWork{x | (uint32_t)q << 8 | (begun[quad] ? 0u : 1u << 12), a, b, off2};
+            else fits = false;
+            ++m;
+            begun[quad] = true;
+        };
+        int st = 0, v = 0;
+        auto put_v = [&]() {
+            const int d = v - dv;
+            if (d >= 0) work(d & 3, (uint32_t)d | 1u << 11, (uint32_t)(k % NST), 0u, 0u);
+            put(v++, 1, true, false, d);
+        };
+        for (int j = 0; j < nu; ++st) {
+            int cnt = 1;
+            const int d0 = j - dj;
+            if (d0 >= 0) {
+                uint32_t bytes = ST_B + 64u * (uint32_t)sh.u_rows(q, j);
+                // (64 elements: one slice a stage, which keeps the schedule at NST entries or more)
+                while (cnt < 4 && j + cnt < nu && sh.ge > 8) {
+                    bytes += ST_B + 64u * (uint32_t)sh.u_rows(q, j + cnt);
+                    if (bytes > ST_BYTES) break;
+                    ++cnt;
+                }
+                // readers of the entry: the quads of its units
+                const uint32_t readers = (uint32_t)((d0 + cnt - 1) / 2 - d0 / 2 + 1);
+                uint32_t o = 0;
+                for (int c = 0; c < cnt; ++c) {
+                    stage_of[d0 + c] = st;
+                    off[d0 + c] = o / 1024u;
+                    where[d0 + c] = (uint32_t)(k % NST) | (o / 1024u) << 4 | (12u / readers) << 12 | (uint32_t)d0 << 16;
+                    o += ST_B + 64u * (uint32_t)sh.u_rows(q, j + c);
+                }
+            }
+            put(j, cnt, false, j == 0, d0);
+            j += cnt;
+            const int done = j - dj;   // diagonal groups issued so far
+            for (int d = d0 < 0 ? 0 : d0; d < done; ++d) {
+                if (!(d & 1)) continue;
+                const int u = d >> 1;
+                const bool same = (where[d] >> 16) == (where[d - 1] >> 16);
+                const bool low = 2 * u < low_groups && 2 * u + 8 >= low_groups;
+                work(u & 3, (uint32_t)u | (low ? 1u << 14 : 0u), where[d - 1], same ? 0u : where[d], off[d]);
+            }
+            if (v < nv) {
+                int at = low_groups > 0 ? low_groups - 1 : -1;   // the diagonal group it waits for
+                if (v >= dv && 4 * (v - dv) + 3 > at) at = 4 * (v - dv) + 3;
+                if (at < 0 || (at < done && st >= stage_of[at] + ADJ_V_LAG)) put_v();
+            }
         }
-        tc::mbar_init(tc::smem_u32(&s_acc_full), 1);
-        tc::mbar_init(tc::smem_u32(&s_acc_empty), 2 * NPROD / 32);
-        tc::mbar_init(tc::smem_u32(&s_acc_low), 2 * NPROD / 32);
-        tc::mbar_init(tc::smem_u32(&s_vready), NPROD / 32);
-        tc::mbar_init(tc::smem_u32(&s_drain), 1);
-        s_err = 0;
+        while (v < nv) put_v();
+        for (int i = 0; i < 4; ++i)
+            if (fits && A->n_work[i] > 0) A->work[i][A->n_work[i] - 1].x |= 1u << 13;   // last of the pass
     }
-    if (warp == 0) tc::tmem_alloc_pair(tc::smem_u32(&s_tmem), A.tmem_cols);
-    tc::fence_before();
-    tc::cluster_sync();   // both CTAs' barriers initialised before any cross-CTA arrival
-    tc::fence_after();
-    const uint32_t tmem = s_tmem;
-    __nv_bfloat16* vimg = A.vimg + (size_t)blockIdx.x * (size_t)(n / 32) * (2 * TP * 32);
-    const int n_pairs = (A.n_tiles + 1) / 2, q0 = (int)blockIdx.x >> 1, nq = (int)gridDim.x >> 1;
-    const int my_items = q0 < n_pairs ? (n_pairs - 1 - q0) / nq + 1 : 0;
-    const int total = my_items * A.F.n * npass * per;
-    const size_t img_u = (size_t)n2 * 16, img_w = (size_t)n * 32;
-    auto stage = [&](int s) { return smem + (size_t)s * ST2_BYTES; };
-    // this CTA's tile of pair item q (the last tile again when the pair has only one)
-    auto tile_of = [&](int q) {
-        const int t = 2 * q + (int)rank;
-        return t < A.n_tiles ? t : A.n_tiles - 1;
-    };
-
-    if (warp == NPROD / 32 + 1) {
-        // ------------------------------ loader (both CTAs) ------------------------------
-        if (lane == 0) {
-            int ql = 0, s = 0, j = 0, fw = 0, pass = 0, q = q0;
-            uint32_t ph = 0, vrp = 0;
-            bool err = false;
-            uint64_t stream_pol;
-            asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(stream_pol));
-            for (; ql < total; ++ql) {
-                if (ql >= NST2 && !tc::mbar_wait(tc::smem_u32(&s_empty[s]), ph ^ 1u, kMaxTries)) {
-                    err = true;
-                    break;
-                }
-                if (s_err) break;
-                const uint32_t mb = tc::smem_u32(&s_full[s]);
-                const int tile = tile_of(q);
-                if (j < nU) {
-                    const uint32_t abytes = TP * 16 * 2;
-                    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(mb),
-                                 "r"(2u * abytes + 2u * (uint32_t)nbk * hb)
-                                 : "memory");
-                    const __nv_bfloat16* asrc =
-                        A.aimg + (size_t)fw * A.aimg_stride + ((size_t)tile * 2 * (n2 / 8) + 2 * j) * 1024;
-                    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint"
-                                 " [%0], [%1], %2, [%3], %4;"
-                                 ::"r"(tc::smem_u32(stage(s))), "l"(asrc), "r"(abytes), "r"(mb), "l"(stream_pol)
-                                 : "memory");
-                    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint"
-                                 " [%0], [%1], %2, [%3], %4;"
-                                 ::"r"(tc::smem_u32(stage(s) + ST2_ALO)), "l"(asrc + (size_t)(n2 / 8) * 1024),
-                                 "r"(abytes), "r"(mb), "l"(stream_pol)
-                                 : "memory");
-                    for (int nb = 0; nb < nbk; ++nb) {
-                        // rows pass ne2 + nb nb_u + rank hrow .. + hrow of both planes
-                        const __nv_bfloat16* bsrc = A.bu + (size_t)fw * A.bu_stride + (size_t)j * 2 * img_u +
-                                                    (size_t)(pass * ne2 + nb * nb_u + (int)rank * hrow) * 16;
-                        const uint32_t dh = tc::smem_u32(stage(s) + ST2_B + (uint32_t)nb * hb);
-                        const uint32_t dl = tc::smem_u32(stage(s) + ST2_B + (uint32_t)(nbk + nb) * hb);
-                        asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                                     ::"r"(dh), "l"(bsrc), "r"(hb), "r"(mb)
-                                     : "memory");
-                        asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                                     ::"r"(dl), "l"(bsrc + img_u), "r"(hb), "r"(mb)
-                                     : "memory");
-                    }
-                } else {
-                    if (j == nU) {
-                        // this CTA's |G|^2 slices of the item are written by its producers
-                        if (!tc::mbar_wait(tc::smem_u32(&s_vready), vrp & 1u, kMaxTries)) {
-                            err = true;
-                            break;
-                        }
-                        ++vrp;
-                    }
-                    const uint32_t wbytes = (uint32_t)wrow * 64u, abytes = 2u * TP * 32 * 2;
-                    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(mb), "r"(wbytes + abytes)
-                                 : "memory");
-                    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                                 ::"r"(tc::smem_u32(stage(s) + ST2_VB)),
-                                 "l"(A.bw + (size_t)fw * A.bw_stride + (size_t)(j - nU) * img_w +
-                                     (size_t)(pass * ne + (int)rank * wrow) * 32),
-                                 "r"(wbytes), "r"(mb)
-                                 : "memory");
-                    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                                 ::"r"(tc::smem_u32(stage(s))), "l"(vimg + (size_t)(j - nU) * (2 * TP * 32)), "r"(abytes),
-                                 "r"(mb)
-                                 : "memory");
-                }
-                if (++s == NST2) { s = 0; ph ^= 1u; }
-                if (++j == per) {
-                    j = 0;
-                    if (++pass == npass) {
-                        pass = 0;
-                        if (++fw == A.F.n) { fw = 0; q += nq; }
-                    }
-                }
-            }
-            if (err || s_err) {
-                s_err = 1;
-                for (int x = (ql > NST2 ? ql - NST2 : 0); x < ql; ++x)
-                    tc::mbar_wait(tc::smem_u32(&s_full[x % NST2]), (uint32_t)(x / NST2) & 1u, kMaxTries);
-            }
-        }
-        __syncwarp();
-    } else if (warp == NPROD / 32 && rank != 0) {
-        // ------------------------------ relay (rank 1) ------------------------------
-        if (lane == 0) {
-            const uint32_t r_pfull = tc::mapa(tc::smem_u32(&s_pfull[0]), 0u);
-            int s = 0;
-            uint32_t ph = 0;
-            for (int ql = 0; ql < total; ++ql) {
-                if (!tc::mbar_wait(tc::smem_u32(&s_full[s]), ph, kMaxTries)) {
-                    s_err = 1;
-                    break;
-                }
-                if (s_err) break;
-                tc::mbar_arrive_remote(r_pfull + 8u * (uint32_t)s);
-                if (++s == NST2) { s = 0; ph ^= 1u; }
-            }
-        }
-        __syncwarp();
-    } else if (warp == NPROD / 32) {
-        // ------------------------------ MMA issuer (rank 0) ------------------------------
-        if (lane == 0) {
-            const uint32_t id_u = tc::idesc_bf16_f32(256, (uint32_t)nb_u);
-            const uint32_t id_v = tc::idesc_bf16_f32(256, (uint32_t)ne);
-            int s = 0, j = 0;
-            uint32_t acce = 0, accl = 0, ph = 0;
-            bool err = false, issued = false;
-            for (int q = 0; q < total && !err; ++q) {
-                if (j == nU) {
-                    // V overwrites the columns of the first N-block of U: both CTAs' part of the U
-                    // epilogue there must be done
-                    if (!tc::mbar_wait_cluster(tc::smem_u32(&s_acc_low), accl & 1u, kMaxTries)) { err = true; break; }
-                    ++accl;
-                } else if (j == 0 && q > 0) {
-                    // a new U phase: both CTAs' V (or U) epilogue must have read the accumulator
-                    if (!tc::mbar_wait_cluster(tc::smem_u32(&s_acc_empty), acce & 1u, kMaxTries)) { err = true; break; }
-                    ++acce;
-                }
-                if (!tc::mbar_wait(tc::smem_u32(&s_full[s]), ph, kMaxTries)) { err = true; break; }
-                if (!tc::mbar_wait_cluster(tc::smem_u32(&s_pfull[s]), ph, kMaxTries)) { err = true; break; }
-                if (s_err) { err = true; break; }
-                tc::fence_after();
-                const uint32_t sa = tc::smem_u32(stage(s)), sal = sa + ST2_ALO, sb = sa + ST2_B;
-                const uint64_t dah = tc::sdesc(sa, 2048, 128), dal = tc::sdesc(sal, 2048, 128);
-                if (j < nU) {
-                    const uint32_t acc = j > 0 ? 1u : 0u;
-                    for (int nb = 0; nb < nbk; ++nb) {
-                        const uint64_t dbh = tc::sdesc(sb + (uint32_t)nb * hb, 128, 256);
-                        const uint64_t dbl = tc::sdesc(sb + (uint32_t)(nbk + nb) * hb, 128, 256);
-                        const uint32_t d = tmem + (uint32_t)(nb * nb_u);
-                        tc::mma_bf16_pair(d, dah, dbh, id_u, acc);
-                        tc::mma_bf16_pair(d, dah, dbl, id_u, 1u);
-                        tc::mma_bf16_pair(d, dal, dbh, id_u, 1u);
-                    }
-                } else {
-#pragma unroll
-                    for (int kh = 0; kh < 2; ++kh) {
-                        const uint64_t vah = tc::sdesc(sa + 256u * kh, 128, 512);
-                        const uint64_t val = tc::sdesc(sa + ST2_VALO + 256u * kh, 128, 512);
-                        const uint64_t vb = tc::sdesc(sa + ST2_VB + 256u * kh, 128, 512);
-                        tc::mma_bf16_pair(tmem, vah, vb, id_v, (j > nU || kh > 0) ? 1u : 0u);
-                        tc::mma_bf16_pair(tmem, val, vb, id_v, 1u);
-                    }
-                }
-                issued = true;
-                tc::commit_pair(tc::smem_u32(&s_empty[s]));
-                if (j == nU - 1 || j == per - 1) tc::commit_pair(tc::smem_u32(&s_acc_full));
-                if (++s == NST2) { s = 0; ph ^= 1u; }
-                if (++j == per) j = 0;
-            }
-            if (err) {
-                s_err = 1;
-                atomicAdd(A.counters + CNT_TC_TIMEOUT, 1u);
-                if (issued) {
-                    tc::commit_pair_local(tc::smem_u32(&s_drain));
-                    tc::mbar_wait(tc::smem_u32(&s_drain), 0u, kMaxTries);
-                }
-            }
-        }
-        __syncwarp();
-    } else {
-        // -------------------------------- producers (both CTAs) --------------------------------
-        const uint32_t p = (uint32_t)(tid & (TP - 1)), h = (uint32_t)(tid / TP);
-        const uint32_t lane_off = (uint32_t)((warp & 3) * 32) << 16;
-        const uint32_t cp = (uint32_t)((lane & 7) + 8 * warp), ch = (uint32_t)(lane >> 3);
-        float2* gs = A.gscr + (size_t)blockIdx.x * n * TP;
-        // the issuer's accumulator barriers (in rank 0), arrived on by both CTAs
-        const uint32_t r_acc_empty = tc::mapa(tc::smem_u32(&s_acc_empty), 0u);
-        const uint32_t r_acc_low = tc::mapa(tc::smem_u32(&s_acc_low), 0u);
-        bool err = false;
-        int qs = 0;
-        uint32_t qph = 0;
-        uint32_t accf = 0;
-        auto slice = [&](auto&& consume) {
-            const int s = qs;
-            if (!err) err = !tc::mbar_wait(tc::smem_u32(&s_full[s]), qph, kMaxTries);
-            err = __any_sync(0xffffffffu, err || s_err != 0);
-            if (!err) consume(stage(s), stage(s) + ST2_ALO);
-            __syncwarp();
-            if (lane == 0 && !err) tc::mbar_arrive(tc::smem_u32(&s_empty[s]));
-            if (++qs == NST2) { qs = 0; qph ^= 1u; }
-        };
-        auto acc_wait = [&]() {
-            if (!err) err = !tc::mbar_wait(tc::smem_u32(&s_acc_full), accf & 1u, kMaxTries);
-            ++accf;
-            err = __any_sync(0xffffffffu, err);
-            tc::fence_after();
-        };
-        auto arrive_issuer = [&](uint32_t caddr) {
-            tc::fence_before();
-            __syncwarp();
-            if (lane == 0 && !err) tc::mbar_arrive_remote(caddr);
-        };
-        for (int q = q0; q < n_pairs; q += nq) {
-            const int tile = tile_of(q);
-            const int px = tile * TP + (int)p;
-            const bool valid = px < G.npix && 2 * q + (int)rank < A.n_tiles;
-            float acc_g = 0.f, acc_h = 0.f;
-            for (int fw = 0; fw < A.F.n; ++fw) {
-                const FreqC fc = A.F.f[fw];
-                float fg_r = 0.f, fg_i = 0.f, fh = 0.f;
-                for (int pass = 0; pass < npass; ++pass) {
-                const int eb0 = pass * ne;
-                for (int j = 0; j < nU; ++j)
-                    slice([&](const unsigned char* ahi, const unsigned char* alo) {
-                        consume_u(j * 8, cp, ch, ahi, alo, gs, vimg, want_h);
-                    });
-                if (want_h) {
-                    asm volatile("fence.proxy.async.global;" ::: "memory");
-                    __syncwarp();
-                    if (lane == 0 && !err) tc::mbar_arrive(tc::smem_u32(&s_vready));
-                }
-                err = tc::named_or(1, NPROD, err);
-                if (err) break;
-                const int nch = 4 * ((ne / 32 - (int)h + 3) / 4);
-                const int nbu = ne2 > 256 ? ne2 / 2 : ne2, ebu = nbu / 2;
-                auto ce0 = [&](int k) { return 32 * ((int)h + 4 * (k >> 2)) + 8 * (k & 3); };
-                auto recol = [&](int e) { return (e / ebu) * nbu + e % ebu; };
-                auto gload = [&](int k, float2 (&g)[8]) {
-                    const int e0 = ce0(k);
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) g[i] = gs[(size_t)(eb0 + e0 + i) * TP + p];
-                };
-                auto gchunk = [&](int k, const float2 (&g)[8], float& ar, float& ai) {
-                    const int e0 = ce0(k);
-                    float vr[8], vi[8];
-                    tc::tmem_ld8(tmem + lane_off + (uint32_t)recol(e0), vr);
-                    tc::tmem_ld8(tmem + lane_off + (uint32_t)(recol(e0) + ebu), vi);
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) {
-                        ar = fmaf(g[i].x, vr[i], fmaf(g[i].y, vi[i], ar));
-                        ai = fmaf(g[i].x, vi[i], fmaf(-g[i].y, vr[i], ai));
-                    }
-                };
-                bool low = false;
-                auto release_low = [&]() {
-                    arrive_issuer(r_acc_low);
-                    low = true;
-                };
-                float2 ga[8], gb[8];
-                if (nch > 0) gload(0, ga);
-                acc_wait();
-                float gr = 0.f, gi = 0.f;
-                if (!err) {
-                    for (int k = 0; k < nch; k += 2) {
-                        if (!low && ce0(k) >= ebu) release_low();
-                        gload(k + 1, gb);
-                        gchunk(k, ga, gr, gi);
-                        if (k + 2 < nch) gload(k + 2, ga);
-                        gchunk(k + 1, gb, gr, gi);
-                    }
-                }
-                if (!low) release_low();
-                if (h > 0) {
-                    s_red[0][h - 1][p] = gr;
-                    s_red[1][h - 1][p] = gi;
-                }
-                err = tc::named_or(1, NPROD, err);
-                if (err) break;
-                if (h == 0) {
-                    fg_r += (gr + s_red[0][0][p] + s_red[0][1][p] + s_red[0][2][p]) * fc.w2;
-                    fg_i += (gi + s_red[1][0][p] + s_red[1][1][p] + s_red[1][2][p]) * fc.w2;
-                }
-                if (!want_h) {
-                    arrive_issuer(r_acc_empty);
-                    continue;
-                }
-                // V slices: the producers only pass the stage barriers (as in the single-CTA kernel)
-                for (int j = 0; j < nV; ++j) slice([&](const unsigned char*, const unsigned char*) {});
-                uint4 qa[2], qb[2];
-                if (nch > 0) g2_load(vimg, eb0 + ce0(0), p, qa);
-                acc_wait();
-                float hh = 0.f;
-                if (!err) {
-                    for (int k = 0; k < nch; k += 2) {
-                        g2_load(vimg, eb0 + ce0(k + 1), p, qb);
-                        h_chunk(tmem + lane_off + (uint32_t)ce0(k), qa, hh);
-                        if (k + 2 < nch) g2_load(vimg, eb0 + ce0(k + 2), p, qa);
-                        h_chunk(tmem + lane_off + (uint32_t)ce0(k + 1), qb, hh);
-                    }
-                }
-                arrive_issuer(r_acc_empty);
-                if (h > 0) s_red[2][h - 1][p] = hh;
-                err = tc::named_or(1, NPROD, err);
-                if (err) break;
-                if (h == 0) fh += (hh + s_red[2][0][p] + s_red[2][1][p] + s_red[2][2][p]) * fc.w4;
-                }   // passes
-                if (err) break;
-                if (h == 0) {
-                    if (valid && A.g_out) A.g_out[(size_t)fw * G.npix + px] = make_float2(fg_r, fg_i);
-                    if (valid && A.h_out) A.h_out[(size_t)fw * G.npix + px] = fh;
-                    acc_g += fg_r;
-                    acc_h += fh;
-                }
-            }
-            if (err) break;
-            if (valid && h == 0) {
-                if (A.gsum) A.gsum[px] = acc_g;
-                if (A.hsum) A.hsum[px] = acc_h;
-            }
-        }
-    }
-    tc::fence_before();
-    tc::cluster_sync();   // the peer is done with this CTA's shared memory and barriers
-    tc::fence_after();
-    if (warp == 0) tc::tmem_dealloc_pair(tmem, A.tmem_cols);
+    A->n_ent = k;
+    return fits && k >= NST;
 }
 }  // namespace
 
@@ -998,10 +758,11 @@ size_t tc_b_images_bytes(int n_elem) {
     return (2 * n) * (2 * n) * 2 * 2 + n * n * 2;   // bu (hi + lo) + bw, bf16
 }
 
-cudaError_t launch_prep_b(int n, const float2* R, const uint8_t* W, void* img, cudaStream_t s) {
-    __nv_bfloat16* bu = (__nv_bfloat16*)img;
-    __nv_bfloat16* bw = bu + (size_t)(2 * n) * (2 * n) * 2;
-    k_prep_b<<<256, 256, 0, s>>>(n, R, W, bu, bw);
+cudaError_t launch_prep_b(int n, int n_freq, const float2* R, const uint8_t* W, void* img, cudaStream_t s) {
+    const AdjShape sh(n);
+    const int npass = n / sh.ne, tri = npass * (npass + 1) / 2;
+    const size_t w_off = (size_t)(2 * n) * (2 * n) * 4;
+    k_prep_b<<<dim3((sh.ge + sh.gv) * tri, n_freq), 128, 0, s>>>(n, R, W, (unsigned char*)img, tc_b_images_bytes(n), w_off);
     return cudaGetLastError();
 }
 
@@ -1040,67 +801,45 @@ __global__ void k_adjoint_sums(const float2* __restrict__ fpart, int n_freq, int
 
 cudaError_t launch_adjoint_tc(const GeoDev& G, const void* aimg, const FreqSet& F, const void* images, float2* gscr,
                               int n_ctas, float2* g_out, float* h_out, float* gsum, float* hsum, uint32_t* counters,
-                              cudaStream_t s, int variant) {
+                              cudaStream_t s) {
     const int n = G.n_elem;
     if (!tc_adjoint_supported(n) || !aimg) return cudaErrorInvalidValue;
+    const AdjShape sh(n);
     TcArgs A;
     A.G = G;
-    A.F = F;
+    A.n_freq = F.n;
+    for (int w = 0; w < F.n; ++w) {
+        A.w2[w] = F.f[w].w2;
+        A.w4[w] = F.f[w].w4;
+    }
     A.aimg = (const __nv_bfloat16*)aimg;
     A.aimg_stride = tc_aimage_elems(n, G.npix);
-    A.bu = (const __nv_bfloat16*)images;
-    A.bu_stride = tc_b_images_bytes(n) / 2;
-    A.bw = A.bu + (size_t)(2 * n) * (2 * n) * 2;
-    A.bw_stride = A.bu_stride;
-    A.gscr = gscr;
-    A.vimg = (__nv_bfloat16*)(gscr + (size_t)RB_TC_MAX_CTAS * n * TP);   // after the G scratch
+    A.bu = (const unsigned char*)images;
+    A.bw = A.bu + (size_t)(2 * n) * (2 * n) * 4;
+    A.b_stride = tc_b_images_bytes(n);
+    A.vimg = (__nv_bfloat16*)gscr;
     A.g_out = g_out;
     A.h_out = h_out;
-    A.gsum = gsum;
-    A.hsum = hsum;
-    A.fpart = nullptr;
-    A.counters = counters;
-    A.n_tiles = (G.npix + TP - 1) / TP;
-    A.n_e = n < 256 ? n : 256;
-    A.want_h = (h_out || hsum) ? 1 : 0;
-    A.npass = n / A.n_e;
-    uint32_t cols = 32;
-    while (cols < (uint32_t)(2 * A.n_e)) cols <<= 1;
-    A.tmem_cols = cols;
-    cudaError_t e;
-    // variant 1: CTA pairs (8 stages of 24 KB); 0 and 2: one CTA per tile (5 stages of 40 KB);
-    // either way most of the SM's shared memory, so one CTA (one TMEM owner) per SM
-    const int n_pairs = (A.n_tiles + 1) / 2;
-    if (variant == 1 && n_ctas >= 2) {
-        const int sm2 = NST2 * (int)ST2_BYTES;
-        const int grid2 = 2 * (n_ctas / 2 < n_pairs ? n_ctas / 2 : n_pairs);
-        if (A.npass == 1) {
-            e = cudaFuncSetAttribute(k_adjoint_tc2<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm2);
-            if (e != cudaSuccess) return e;
-            k_adjoint_tc2<false><<<grid2, NTHR_A, sm2, s>>>(A);
-        } else {
-            e = cudaFuncSetAttribute(k_adjoint_tc2<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm2);
-            if (e != cudaSuccess) return e;
-            k_adjoint_tc2<true><<<grid2, NTHR_A, sm2, s>>>(A);
-        }
-        return cudaGetLastError();
-    }
     // the CTAs take (tile, frequency) items in turn, so the sums over the set go through
     // the per-frequency buffer that follows the per-CTA scratch in the workspace
-    if (gsum || hsum)
-        A.fpart = (float2*)(A.vimg + (size_t)RB_TC_MAX_CTAS * n * 256);
+    A.fpart = (gsum || hsum) ? (float2*)(A.vimg + (size_t)RB_TC_MAX_CTAS * 2 * n * 256) : nullptr;
+    A.counters = counters;
+    A.n_tiles = (G.npix + TP - 1) / TP;
+    A.want_h = (h_out || hsum) ? 1 : 0;
+    // V beside U where TMEM's 512 columns hold both, else in the first columns of U
+    A.v_col = 3 * sh.ne <= 512 ? 2u * (uint32_t)sh.ne : 0u;
+    A.low_groups = A.v_col || !A.want_h ? 0 : sh.ne / 16;
+    const int need = A.v_col ? 3 * sh.ne : 2 * sh.ne;
+    A.tmem_cols = 32;
+    while (A.tmem_cols < (uint32_t)need) A.tmem_cols <<= 1;
+    if (!adj_schedule(sh, A.want_h != 0, A.low_groups, &A)) return cudaErrorInvalidValue;
+    // most of the SM's shared memory, so one CTA (one TMEM owner) per SM
     const int sm = NST * (int)ST_BYTES;
     const int n_items = A.n_tiles * F.n;
     const int grid = n_ctas < n_items ? n_ctas : n_items;
-    if (A.npass == 1) {
-        e = cudaFuncSetAttribute(k_adjoint_tc<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-        if (e != cudaSuccess) return e;
-        k_adjoint_tc<false><<<grid, NTHR_A, sm, s>>>(A);
-    } else {
-        e = cudaFuncSetAttribute(k_adjoint_tc<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-        if (e != cudaSuccess) return e;
-        k_adjoint_tc<true><<<grid, NTHR_A, sm, s>>>(A);
-    }
+    cudaError_t e = cudaFuncSetAttribute(k_adjoint_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+    if (e != cudaSuccess) return e;
+    k_adjoint_tc<<<grid, NTHR_A, sm, s>>>(A);
     e = cudaGetLastError();
     if (e != cudaSuccess || !A.fpart) return e;
     k_adjoint_sums<<<(G.npix + 255) / 256, 256, 0, s>>>(A.fpart, F.n, G.npix, gsum, hsum);

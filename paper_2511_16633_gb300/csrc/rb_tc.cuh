@@ -109,88 +109,6 @@ __device__ __forceinline__ void mbar_arrive_cnt(uint32_t mbar, uint32_t count) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0], %1;" ::"r"(mbar), "r"(count) : "memory");
 }
 
-// ---------------------------------------------------------------------------
-// CTA pairs (a cluster of two CTAs, cta_group::2): one MMA over both CTAs' shared
-// memory (A: M / 2 rows from each CTA; B: N / 2 columns from each), accumulating in
-// both CTAs' TMEM (M / 2 lanes each), issued by the pair's rank-0 CTA.
-// ---------------------------------------------------------------------------
-__device__ __forceinline__ uint32_t cluster_ctarank() {
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-
-// All threads of both CTAs of the cluster (release / acquire at cluster scope).
-__device__ __forceinline__ void cluster_sync() {
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-
-// The shared::cluster address of this CTA's shared variable `saddr` in CTA `rank` of the cluster.
-__device__ __forceinline__ uint32_t mapa(uint32_t saddr, uint32_t rank) {
-    uint32_t r;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(saddr), "r"(rank));
-    return r;
-}
-
-// One arrival on an mbarrier of another CTA of the cluster (shared::cluster address).
-__device__ __forceinline__ void mbar_arrive_remote(uint32_t caddr) {
-    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(caddr) : "memory");
-}
-
-// Bounded wait with cluster-scope acquire (for barriers that other CTAs arrive on).
-__device__ __forceinline__ bool mbar_wait_cluster(uint32_t mbar, uint32_t parity, uint32_t max_tries) {
-    for (uint32_t i = 0; i < max_tries; ++i) {
-        uint32_t ok;
-        asm volatile(
-            "{\n\t.reg .pred p;\n\t"
-            "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
-            "selp.u32 %0, 1, 0, p;\n\t}"
-            : "=r"(ok)
-            : "r"(mbar), "r"(parity)
-            : "memory");
-        if (ok) return true;
-    }
-    return false;
-}
-
-__device__ __forceinline__ void mma_bf16_pair(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accum) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-        :
-        : "r"(d_tmem), "l"(a), "l"(b), "r"(idesc), "r"(accum)
-        : "memory");
-}
-
-// Completion of the pair's MMAs issued so far, arriving on the mbarrier at the same
-// shared-memory offset in both CTAs.
-__device__ __forceinline__ void commit_pair(uint32_t mbar) {
-    asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
-                 ::"r"(mbar), "h"((unsigned short)3)
-                 : "memory");
-}
-
-// The same, arriving on this CTA's mbarrier only.
-__device__ __forceinline__ void commit_pair_local(uint32_t mbar) {
-    asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(mbar) : "memory");
-}
-
-// TMEM of a CTA pair: one warp of each CTA allocates (and later frees) the same columns.
-__device__ __forceinline__ void tmem_alloc_pair(uint32_t slot_saddr, uint32_t ncols) {
-    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(slot_saddr), "r"(ncols)
-                 : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
-}
-__device__ __forceinline__ void tmem_dealloc_pair(uint32_t taddr, uint32_t ncols) {
-    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
-}
-
-// Barrier over the first `nthreads` threads of the CTA (a multiple of 32) on hardware barrier `id`.
-__device__ __forceinline__ void named_sync(uint32_t id, uint32_t nthreads) {
-    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
-}
-
 // Barrier over the first `nthreads` threads that also ORs a predicate across them.
 __device__ __forceinline__ bool named_or(uint32_t id, uint32_t nthreads, bool v) {
     uint32_t r;
@@ -221,12 +139,53 @@ __device__ __forceinline__ bool mbar_wait(uint32_t mbar, uint32_t parity, uint32
     return false;
 }
 
-// One thread: arm the barrier for `bytes` of asynchronous copy and issue a 1-D bulk
-// copy global -> shared that completes them (addresses 16-byte aligned, bytes % 16 == 0).
-__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t mbar) {
+// The issuing warps (loaders, MMA issuers) run their loops with all 32 lanes, on values the
+// compiler can see to be the same in every lane, and predicate only the issuing
+// instructions on one elected lane: descriptors, addresses and barriers then live in
+// uniform registers and the waits of the other lanes do not serialise.  Measured on the
+// adjoint (256 elements, 512 x 512 pixels, one frequency, no Hessian): 340 us with the
+// loops in a one-lane branch, 272 us so.  Votes keep the loops' exits warp-uniform.
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "elect.sync _|p, 0xffffffff;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(p));
+    return p != 0;
+}
+
+// Bounded wait of a whole warp (warp-uniform result): false on timeout or once *err is raised.
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t mbar, uint32_t parity, uint32_t max_tries, const volatile int* err) {
+    for (uint32_t i = 0; i < max_tries; ++i) {
+        uint32_t ok;
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(ok)
+            : "r"(mbar), "r"(parity)
+            : "memory");
+        if (__all_sync(0xffffffffu, ok != 0)) return true;
+        if (__any_sync(0xffffffffu, *err != 0)) return false;
+    }
+    return false;
+}
+
+// One thread: arm the barrier for `bytes` of asynchronous copies.
+__device__ __forceinline__ void bulk_arm(uint32_t mbar, uint32_t bytes) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(mbar), "r"(bytes) : "memory");
+}
+// One thread: a 1-D bulk copy global -> shared that completes `bytes` on the armed barrier
+// (addresses 16-byte aligned, bytes % 16 == 0); with an L2 cache policy below.
+__device__ __forceinline__ void bulk_copy(uint32_t dst, const void* src, uint32_t bytes, uint32_t mbar) {
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
                  "l"(src), "r"(bytes), "r"(mbar)
+                 : "memory");
+}
+__device__ __forceinline__ void bulk_copy_hint(uint32_t dst, const void* src, uint32_t bytes, uint32_t mbar, uint64_t policy) {
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1], %2, [%3], %4;"
+                 ::"r"(dst), "l"(src), "r"(bytes), "r"(mbar), "l"(policy)
                  : "memory");
 }
 

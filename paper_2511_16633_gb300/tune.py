@@ -3,9 +3,8 @@
 The rasteriser of the gridding has two work mappings, warps along the ray tubes or
 across them, whose speed depends on how wide the tubes are against the pixels and on
 how much the medium bends them; the library's rule picks by tube width alone.  The
-tensor-core adjoint runs either on one CTA per pixel tile or on CTA pairs sharing each
-MMA (cta_group::2), which halves the shared-memory traffic of the S operand per CTA.
-The choices do not change the results, so only their time differs, and that is
+tensor-core adjoint has one form, one CTA per pixel tile; the field that chose CTA pairs
+before is still accepted, and its values are still told apart here.  The choices do not change the results, so only their time differs, and that is
 measured here: for one problem, ``tune_update`` times the updates per candidate on
 the caller's own data (a warm-up run, then ``reps`` timed ones, each from a scratch
 copy of c, with CUDA events on a private stream; a whole sweep over the problem's
@@ -27,7 +26,7 @@ ADJOINT = {rb.RB_TUNE_ADJ_SINGLE: "adjoint one CTA per tile", rb.RB_TUNE_ADJ_PAI
 
 def candidates(prec: int):
     """The tune values tried for a precision: both raster mappings, and on the tensor-core
-    path both forms of the adjoint."""
+    path both values of the adjoint's field."""
     if prec == rb.RB_PREC_BF16X3:
         return tuple(r | a for a in ADJOINT for r in RASTER)
     return tuple(RASTER)
