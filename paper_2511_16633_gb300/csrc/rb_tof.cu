@@ -38,8 +38,8 @@ __device__ __forceinline__ float fp_diff(float vh, float vl, float oh, float ol)
 }
 
 __device__ __forceinline__ Vtx load_vtx(const Vtx* __restrict__ p) {
-    const float4* q = reinterpret_cast<const float4*>(p);
-    const float4 a = __ldg(q), b = __ldg(q + 1);
+    float4 a, b;
+    ldg32(p, a, b);
     return Vtx{a.x, a.y, a.z, a.w, b.x, b.y, b.z, __float_as_int(b.w)};
 }
 

@@ -57,9 +57,14 @@ __device__ __forceinline__ void sample(const GeoDev& G, const float4* __restrict
     const float fi = fminf(floorf(u), G.fxmax - 1.f), fj = fminf(floorf(v), G.fymax - 1.f);
     const float fu = u - fi, fv = v - fj;
     if (fi != cc.fi || fj != cc.fj) {
+        // the lanes' records are on lines of their own, so each load costs the LSU a wavefront
+        // per lane whatever its width: four 32-byte loads instead of seven of 16 bytes
         const float4* p = cells + ((size_t)(int)fj * (size_t)(G.nx - 1) + (size_t)(int)fi) * 8;
-#pragma unroll
-        for (int k = 0; k < 7; ++k) cc.r[k] = __ldg(p + k);
+        float4 pad;
+        ldg32(p, cc.r[0], cc.r[1]);
+        ldg32(p + 2, cc.r[2], cc.r[3]);
+        ldg32(p + 4, cc.r[4], cc.r[5]);
+        ldg32(p + 6, cc.r[6], pad);
         cc.fi = fi;
         cc.fj = fj;
     }
@@ -312,9 +317,7 @@ __device__ __forceinline__ void udivmod(uint32_t q, uint32_t d, uint32_t m, uint
 __device__ __forceinline__ size_t vidx(const GeoDev& G, int t, int k, int i) { return vtx_index(G, t, k, i); }
 
 __device__ __forceinline__ void put_vtx(Vtx* dst, const Vtx& v) {
-    float4* d = reinterpret_cast<float4*>(dst);
-    d[0] = make_float4(v.xh, v.xl, v.yh, v.yl);
-    d[1] = make_float4(v.t, v.q, v.l, __int_as_float(v.k));
+    stg32(dst, make_float4(v.xh, v.xl, v.yh, v.yl), make_float4(v.t, v.q, v.l, __int_as_float(v.k)));
 }
 
 // One thread per ray: RK4 from the element to the ring, the end record, and (when
@@ -490,8 +493,8 @@ __device__ __forceinline__ int last_vertex(const GeoDev& G, const rb_ray_end* __
 }
 
 __device__ __forceinline__ Vtx get_vtx(const Vtx* __restrict__ src) {
-    const float4* s = reinterpret_cast<const float4*>(src);
-    const float4 a = __ldg(s), b = __ldg(s + 1);
+    float4 a, b;
+    ldg32(src, a, b);
     return Vtx{a.x, a.y, a.z, a.w, b.x, b.y, b.z, __float_as_int(b.w)};
 }
 
