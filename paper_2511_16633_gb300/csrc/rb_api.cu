@@ -318,7 +318,7 @@ rb_status gradient_stages(const GeoDev& G, const FreqSet& F, const Ws& W, float*
                                 nullptr, nullptr, W.at<float>(W.L.gsum), W.at<float>(W.L.hsum), cnt, s));
     } else {
         RB_CU(launch_adjoint_simt(G, tables, c, F, R, wts, nullptr, nullptr, W.at<float>(W.L.gsum),
-                                  W.at<float>(W.L.hsum), cnt, s));
+                                  W.at<float>(W.L.hsum), W.at<void>(W.L.sym), s));
     }
     RB_CU(mark(RB_STAGE_ADJOINT, 1));
     return RB_OK;
@@ -355,7 +355,8 @@ size_t rb_ws_layout(const rb_geometry* g, int n_freq, rb_precision prec, WsLayou
     L->hsum = o; o = align256(o + npix * 4);
     L->pdir = o; o = align256(o + npix * 4);
     L->part = o; o = align256(o + (size_t)(RB_MAX_FREQ + 2) * 256 * 8);
-    L->fwd = o; o = align256(o + (tcp ? 0 : (size_t)rb_fwd_chunks_for((int)npix) * ne * ne * 8));
+    L->fwd = o; o = align256(o + (tcp ? 0 : (size_t)rb_fwd_chunks_for(g->n_elem, (int)npix) * ne * ne * 8));
+    L->sym = o; o = align256(o + (tcp ? 0 : nf * simt_sym_bytes(g->n_elem)));
     L->tcimg = o; o = align256(o + (tcp ? (size_t)n_freq * tc_b_images_bytes(g->n_elem) : 0));
     // two sets of |G|^2 A slices (bf16 hi and lo) per persistent CTA, then (Re g, H)
     // of each frequency of the set for the adjoint's sums over the set
@@ -500,7 +501,7 @@ rb_status rb_born_forward(const rb_geometry* geom, const rb_cell* tables, const 
     uint32_t* cnt = W.at<uint32_t>(W.L.counters);
     const GeoDev G = make_geo(geom, exy);
     const FreqC F = make_freq(geom, f_hz);
-    const int nch = rb_fwd_chunks_for(G.npix);
+    const int nch = rb_fwd_chunks_for(G.n_elem, G.npix);
     RB_CU(launch_elem_positions(G, exy, s));
     if (prec == RB_PREC_BF16X3) {
         RB_CU(cudaMemsetAsync(cnt, 0, CNT_N * 4, s));
@@ -511,7 +512,7 @@ rb_status rb_born_forward(const rb_geometry* geom, const rb_cell* tables, const 
         RB_CU(launch_forward_tc(G, W.at<void>(W.L.aimg), F, m, W.at<float>(W.L.tcfwd), tc_ctas(), (float2*)d_out,
                                 nullptr, nullptr, cnt, s));
     } else {
-        RB_CU(launch_forward_simt(G, tables, c, F, m, W.at<float2>(W.L.fwd), nch, s));
+        RB_CU(launch_forward_simt(G, tables, c, F, m, W.at<float2>(W.L.gkeys), W.at<float2>(W.L.fwd), nch, s));
         RB_CU(launch_forward_reduce(G, F, W.at<float2>(W.L.fwd), nch, (float2*)d_out, nullptr, nullptr, s));
     }
     return RB_OK;
@@ -545,7 +546,7 @@ rb_status rb_born_adjoint(const rb_geometry* geom, const rb_cell* tables, const 
                                 (float2*)g_out, hdiag_out, nullptr, nullptr, cnt, s));
     } else {
         RB_CU(launch_adjoint_simt(G, tables, c, F, (const float2*)resid, w, (float2*)g_out, hdiag_out, nullptr,
-                                  nullptr, nullptr, s));
+                                  nullptr, W.at<void>(W.L.sym), s));
     }
     return RB_OK;
 }
@@ -575,7 +576,7 @@ rb_status rb_hf_update(const rb_geometry* geom, float* c_inout, const float* alp
     float* pdir = W.at<float>(W.L.pdir);
     double* part = W.at<double>(W.L.part);
     float2* fwd = W.at<float2>(W.L.fwd);
-    const int nch = rb_fwd_chunks_for(G.npix);
+    const int nch = rb_fwd_chunks_for(G.n_elem, G.npix);
     RB_CU(mark(RB_STAGE_DIRECTION, 0));
     RB_CU(launch_update(G, c_inout, gsum, hsum, pdir, dc_out, part, dbl, cnt, diag_out, params->eps_rel,
                         params->step_mode, 0, s));
@@ -600,7 +601,7 @@ rb_status rb_hf_update(const rb_geometry* geom, float* c_inout, const float* alp
                 if (w == n_freq - 1) RB_CU(cudaStreamWaitEvent(s, ss->red[w & 1], 0));   // the last reduce (the
                                                                                           // others precede it)
             } else {
-                RB_CU(launch_forward_simt(G, tables, c_inout, F.f[w], pdir, fwd, nch, s));
+                RB_CU(launch_forward_simt(G, tables, c_inout, F.f[w], pdir, W.at<float2>(W.L.gkeys), fwd, nch, s));
                 RB_CU(launch_forward_reduce(G, F.f[w], fwd, nch, nullptr, wts + (size_t)w * ne2,
                                             part + (size_t)w * 256, s));
             }
@@ -648,7 +649,7 @@ rb_status rb_cg_update(const rb_geometry* geom, float* c_inout, const float* alp
     // the residuals are consumed by the gradient: their buffer holds B_w p from here on
     float2* d = W.at<float2>(W.L.pray);
     const bool tc = prec == RB_PREC_BF16X3;
-    const int nch = rb_fwd_chunks_for(G.npix);
+    const int nch = rb_fwd_chunks_for(G.n_elem, G.npix);
     RB_CU(mark(RB_STAGE_DIRECTION, 0));
     RB_CU(launch_cg_init(G, gsum, hsum, precond, x, r, p, part, dbl, params->eps_rel, s));
     RB_CU(mark(RB_STAGE_DIRECTION, 1));
@@ -662,7 +663,7 @@ rb_status rb_cg_update(const rb_geometry* geom, float* c_inout, const float* alp
                                         F.f[w], p, W.at<float>(W.L.tcfwd), tc_ctas(), dw, wts + (size_t)w * ne2,
                                         part + (size_t)w * 256, cnt, s));
             } else {
-                RB_CU(launch_forward_simt(G, tables, c_inout, F.f[w], p, W.at<float2>(W.L.fwd), nch, s));
+                RB_CU(launch_forward_simt(G, tables, c_inout, F.f[w], p, W.at<float2>(W.L.gkeys), W.at<float2>(W.L.fwd), nch, s));
                 RB_CU(launch_forward_reduce(G, F.f[w], W.at<float2>(W.L.fwd), nch, dw, wts + (size_t)w * ne2,
                                             part + (size_t)w * 256, s));
             }
@@ -674,7 +675,7 @@ rb_status rb_cg_update(const rb_geometry* geom, float* c_inout, const float* alp
             RB_CU(launch_adjoint_tc(G, W.at<void>(W.L.aimg), F, W.at<void>(W.L.tcimg), W.at<float2>(W.L.gscr),
                                     tc_ctas(), nullptr, nullptr, q, nullptr, cnt, s));
         } else {
-            RB_CU(launch_adjoint_simt(G, tables, c_inout, F, d, wts, nullptr, nullptr, q, nullptr, cnt, s));
+            RB_CU(launch_adjoint_simt(G, tables, c_inout, F, d, wts, nullptr, nullptr, q, nullptr, W.at<void>(W.L.sym), s));
         }
         RB_CU(launch_cg_step(G, hsum, precond, k, x, r, p, q, vpart, dbl, s));
     }

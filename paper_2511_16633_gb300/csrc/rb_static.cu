@@ -68,14 +68,14 @@ extern "C" rb_status rb_born_forward_noalloc(const rb_geometry* geom, const rb_c
     if (scratch_address(&base) != cudaSuccess) return RB_ERR_CUDA;
     float4* exy = (float4*)base;
     float2* partial = (float2*)((char*)base + kElemBytes);
-    int nch = rb_fwd_chunks_for(geom->nx * geom->ny);
+    int nch = rb_fwd_chunks_for(geom->n_elem, geom->nx * geom->ny);
     const int fit = (int)(kPartialBytes / per_chunk);
     if (nch > fit) nch = fit;
     const GeoDev G = rb_make_geo(geom, exy);
     const FreqC F = rb_make_freq(geom, f_hz);
     cudaStream_t s = (cudaStream_t)stream;
     if (launch_elem_positions(G, exy, s) != cudaSuccess) return RB_ERR_CUDA;
-    if (launch_forward_simt(G, tables, c, F, m, partial, nch, s) != cudaSuccess) return RB_ERR_CUDA;
+    if (launch_forward_simt(G, tables, c, F, m, nullptr, partial, nch, s) != cudaSuccess) return RB_ERR_CUDA;
     if (launch_forward_reduce(G, F, partial, nch, (float2*)d_out, nullptr, nullptr, s) != cudaSuccess)
         return RB_ERR_CUDA;
     return RB_OK;

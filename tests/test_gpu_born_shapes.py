@@ -81,3 +81,42 @@ def test_tensor_core_adjoint_of_asymmetric_weights(dev, n, nx, ny):
         assert _rel(out, ref_g) <= 3e-5
         if want_h:
             assert _rel(h, ref_h) <= 2e-5
+
+
+# plain FP32: blocks of 32 elements (odd rings, the largest), one and several pixel tiles
+@pytest.mark.parametrize("n,nx,ny", [(2, 20, 21), (31, 40, 37), (33, 64, 65), (100, 50, 51), (150, 61, 60), (512, 30, 33)])
+def test_plain_adjoint_of_asymmetric_weights(dev, n, nx, ny):
+    geom, tab, c, G, f, g = _problem(dev, n, nx, ny)
+    S = torch.view_as_complex(torch.randn((n, n, 2), generator=g, device=dev)).contiguous()
+    W = (torch.rand((n, n), generator=g, device=dev) < 0.7).to(torch.uint8).contiguous()
+    W[0, 1] = 1
+    ws = rb.workspace(geom, 1, rb.RB_PREC_FP32, dev)
+    w2 = (2 * math.pi * f) ** 2
+    Sw = S.to(torch.complex128) * W
+    P = G.abs().square()
+    out = torch.full((nx * ny,), float("nan"), dtype=torch.complex64, device=dev)
+    h = torch.full((nx * ny,), float("nan"), device=dev)
+    rb.rb_born_adjoint(geom, tab, c, f, S, W, out, ws, h, rb.RB_PREC_FP32)
+    assert _rel(out, w2 * (G.conj() * (Sw @ G.conj())).sum(0)) <= 1e-5
+    assert _rel(h, w2 * w2 * (P * (W.double() @ P)).sum(0)) <= 1e-5
+
+
+# tensor cores: one to 40 pairs of row block and column group, fewer and more slices than
+# splits; plain FP32: one to 36 tile pairs, one chunk and many
+@pytest.mark.parametrize("prec,n,nx,ny", [("tc", 64, 20, 21), ("tc", 64, 64, 64), ("tc", 128, 97, 60), ("tc", 192, 70, 71),
+                                          ("tc", 256, 40, 33), ("tc", 256, 160, 149), ("tc", 512, 71, 70), ("tc", 768, 33, 35),
+                                          ("tc", 1024, 40, 41), ("fp32", 2, 20, 21), ("fp32", 63, 64, 64), ("fp32", 65, 33, 20),
+                                          ("fp32", 150, 120, 121), ("fp32", 512, 30, 33)])
+def test_forward_shapes(dev, prec, n, nx, ny):
+    geom, tab, c, G, f, g = _problem(dev, n, nx, ny)
+    m = 1e-9 * torch.randn(nx * ny, generator=g, device=dev)
+    p = rb.RB_PREC_BF16X3 if prec == "tc" else rb.RB_PREC_FP32
+    ws = rb.workspace(geom, 1, p, dev)
+    ref = (2 * math.pi * f) ** 2 * (G * m.double()) @ G.T
+    d = torch.full((n, n), float("nan"), dtype=torch.complex64, device=dev)
+    rb.rb_born_forward(geom, tab, c, f, m, d, ws, p)
+    assert _rel(d, ref) <= (3e-5 if prec == "tc" else 1e-5)
+    if prec == "fp32":   # the same without a workspace: G synthesised per tile pair
+        d.fill_(float("nan"))
+        rb.rb_born_forward_noalloc(geom, tab, c, f, m, d)
+        assert _rel(d, ref) <= 1e-5
