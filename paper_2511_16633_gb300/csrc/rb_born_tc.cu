@@ -57,9 +57,9 @@ struct AdjShape {
 // each slice holding the rows its pass multiplies and the slices packed in pass order:
 //   bu: [pass, slice of 8 elements r][hi|lo][rows e' x 16]   (tile16_offset)
 //   bw: [pass, slice of 32 elements r][rows e x 32]           (chunk_offset)
-// CTA (slice, frequency); a thread takes one row's 4 (U) or 8 (V) elements r and writes
-// its 16-byte core rows: 256 elements, 4 frequencies in one launch (four launches of
-// 6.5 us each, one bf16 per store, before).
+// CTA (slice, frequency, quarter); a thread takes one row's 4 (U) or 8 (V) elements r and
+// writes its 16-byte core rows; one launch for all frequencies (four launches of 6.5 us
+// each, one bf16 per store, before).
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(128) k_prep_b(int n, const float2* __restrict__ Rs, const uint8_t* __restrict__ Ws,
                                                 unsigned char* __restrict__ img, size_t img_stride, size_t w_off) {
@@ -75,7 +75,7 @@ __global__ void __launch_bounds__(128) k_prep_b(int n, const float2* __restrict_
     if (!is_v) {
         const int rows = sh.u_rows(q, j), cnt = rows / 2, e0 = (q + 1) * sh.ne - cnt;
         unsigned char* dst = out + sh.u_off(q, j);
-        for (int idx = threadIdx.x; idx < 2 * cnt; idx += blockDim.x) {
+        for (int idx = blockIdx.z * blockDim.x + threadIdx.x; idx < 2 * cnt; idx += gridDim.z * blockDim.x) {
             const int el = idx % cnt, kc = idx / cnt, e = e0 + el;
             uint32_t rh[4], rl[4], ih[4], il[4];
 #pragma unroll
@@ -106,7 +106,7 @@ __global__ void __launch_bounds__(128) k_prep_b(int n, const float2* __restrict_
     } else {
         const int rows = sh.v_rows(q, j), e0 = (q + 1) * sh.ne - rows;
         unsigned char* dst = out + w_off + sh.v_off(q, j);
-        for (int idx = threadIdx.x; idx < 4 * rows; idx += blockDim.x) {
+        for (int idx = blockIdx.z * blockDim.x + threadIdx.x; idx < 4 * rows; idx += gridDim.z * blockDim.x) {
             const int el = idx % rows, core = idx / rows, e = e0 + el;
             uint32_t v[8];
 #pragma unroll
@@ -185,7 +185,7 @@ namespace {
 // Pipeline shapes of the tensor-core kernels.
 constexpr int NPROD = 512;                   // adjoint epilogue threads: four quads of 128 (thread = pixel)
 constexpr int NTHR_A = NPROD + 64;           // + MMA warp + loader warp
-constexpr int NPROD_F = 256;                 // forward producer threads: two per A row
+constexpr int NPROD_F = 512;                 // forward producer threads: four groups of one per A row
 constexpr int NTHR_F = NPROD_F + 64;
 constexpr int NST = 5;                       // pipeline stages
 constexpr uint32_t ST_BYTES = 40u * 1024u;   // A hi (4 KB) + A lo (4 KB) + B (<= 32 KB)
@@ -762,7 +762,7 @@ cudaError_t launch_prep_b(int n, int n_freq, const float2* R, const uint8_t* W, 
     const AdjShape sh(n);
     const int npass = n / sh.ne, tri = npass * (npass + 1) / 2;
     const size_t w_off = (size_t)(2 * n) * (2 * n) * 4;
-    k_prep_b<<<dim3((sh.ge + sh.gv) * tri, n_freq), 128, 0, s>>>(n, R, W, (unsigned char*)img, tc_b_images_bytes(n), w_off);
+    k_prep_b<<<dim3((sh.ge + sh.gv) * tri, n_freq, 4), 128, 0, s>>>(n, R, W, (unsigned char*)img, tc_b_images_bytes(n), w_off);
     return cudaGetLastError();
 }
 
@@ -854,79 +854,86 @@ cudaError_t launch_adjoint_tc(const GeoDev& G, const void* aimg, const FreqSet& 
 //   Re d = D[2e][2r] - D[2e+1][2r+1],  Im d = -(D[2e][2r+1] + D[2e+1][2r]).
 // Both operands come from the adjoint's A image (layout of aimg_put4), read MN-major:
 // a core matrix there is 8 pixels (K) x 8 consecutive r' (16 bytes each), and a
-// 16-pixel K slice of all r' rows is one 2-D TMA box per plane.  CTA (i, s):
-// 128-row block i of D over pixel split s, the needed column blocks in TMEM;
-// column blocks below the diagonal are skipped (symmetry).  Partial D blocks go to
+// 16-pixel K slice of up to 32 rows of 8 r' is one 2-D TMA box per plane.  CTA (pair, s):
+// the pair's 128-row block i of D and column range over pixel split s, accumulated in
+// TMEM; columns left of the row block are skipped (symmetry).  Partial D blocks go to
 // global memory and a second kernel sums the splits in order.
 // ===========================================================================
 namespace {
 
 constexpr int FMAXB = 16;  // max row blocks (2n / 128, n <= 1024)
-constexpr int FMAXG = 4;   // max column groups of two 256-column blocks (2n / 512)
+constexpr int FMAXG = 4;   // max column groups of 512 columns (2n / 512)
 constexpr int FMAXP = 40;  // max (row block, column group) pairs (40 for n = 1024)
-constexpr int FBOX_MAX = 32;   // rows (of 8 r') per TMA box, at most
+constexpr int FMAXST = 12; // max pipeline stages
+constexpr double FWD_MIN_KB = 80.0;   // see make_fwd_args
+constexpr int FBOX = 32;   // rows (of 8 r') per TMA box (16 where fewer are left)
 constexpr uint32_t ST_FB = 8192u;   // forward stage: A hi (4 KB), A lo (4 KB), then B hi and B lo
 
 struct FwdArgs {
     GeoDev G;
-    FreqC F;
+    float w2;
     const float* m;
     float* partial;            // [cta][128][2n] fp32 (only needed columns written)
     int n_mb;                  // row blocks
-    int nbn, nb;               // column blocks and their width
-    // work pairs: row block p_i with the column blocks [p_jb, p_je) (at most two, so the
-    // accumulators fit TMEM), each split over pixel ranges
+    // work pairs: row block p_i with the columns [p_c0, p_c1) (at most 512, so the accumulators
+    // fit TMEM), each split over pixel ranges
     int n_pairs;
-    int p_i[FMAXP], p_jb[FMAXP], p_je[FMAXP];
+    int p_i[FMAXP], p_c0[FMAXP], p_c1[FMAXP];
     int splits[FMAXP];         // splits per pair
     int cta0[FMAXP + 1];       // first CTA of each pair
-    int pidx[FMAXB][FMAXG];    // pair of (row block, column group of two blocks)
+    int pidx[FMAXB][FMAXG];    // pair of (row block, column group)
     uint32_t tmem_cols;
     uint32_t* counters;
-    int fbox;                  // rows per TMA box of the B rows: divides every pair's loaded rows
 };
 
-__host__ __device__ __forceinline__ int jmin_of(int i, int nb) { return (128 * i) / nb; }
+// Stages of a pair of `cols` columns: as many as 200 KB hold, at most FMAXST.
+__host__ __device__ __forceinline__ int fwd_stages(int cols) {
+    const int k = (200 * 1024) / ((int)ST_FB + 64 * cols);
+    return k < FMAXST ? k : FMAXST;
+}
 
 // Forward kernel: warp-specialised pipeline over K = 16 pixel slices.
-//   warps 0..7  producers: thread u takes the 16-byte row (8 r', one pixel) u of the
-//               row block's A slice: B rows 128 i .. 128 i + 127 scaled by m(x) and
-//               re-split into hi / lo, once the slice's B has landed; then the epilogue;
-//   warp 8      MMA issuer; warp 9 loader (TMA boxes of the rows [col0, 2n) of the
-//               slice, hi and lo planes).
+//   warps 0..15 producers, four groups of 128 threads, each on every fourth slice (a slice's
+//               way through a group is mostly latency): thread u of a group takes the 16-byte
+//               rows (8 r', one pixel) u and u + 128 of the row block's A slice: rows 128 i ..
+//               128 i + 127 scaled by m(x) and re-split into hi / lo, once the slice has
+//               landed; then the epilogue;
+//   warp 16     MMA issuer; warp 17 loader (TMA boxes of the columns' rows of the slice, hi
+//               and lo planes), both warp-uniform.
 // SEP: some pairs load their row block's own rows separately (rings above 256 elements);
 // without it every pair finds them among its B rows and the test compiles away.
 template <bool SEP>
-__global__ void __launch_bounds__(NTHR_F, 1) k_forward_tc(FwdArgs A, const __grid_constant__ CUtensorMap tmap,
+__global__ void __launch_bounds__(NTHR_F, 1) k_forward_tc(const __grid_constant__ FwdArgs A, const __grid_constant__ CUtensorMap tmap,
                                                          const __grid_constant__ CUtensorMap tmap16) {
     extern __shared__ __align__(1024) unsigned char smem[];
-    __shared__ uint64_t s_full_a[NST], s_full_b[NST], s_empty[NST], s_acc_full;
+    __shared__ uint64_t s_full_a[FMAXST], s_full_b[FMAXST], s_empty[FMAXST], s_acc_full;
     __shared__ uint32_t s_tmem;
     __shared__ volatile int s_err;
     const GeoDev& G = A.G;
     const int n = G.n_elem, n2 = 2 * n;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     int pq = 0;
     while (pq + 1 < A.n_pairs && (int)blockIdx.x >= A.cta0[pq + 1]) ++pq;
-    const int i = A.p_i[pq], jb = A.p_jb[pq], je = A.p_je[pq];
+    const int i = A.p_i[pq], col0 = A.p_c0[pq], cols = A.p_c1[pq] - col0;   // needed columns (= B rows loaded)
     const int sp = (int)blockIdx.x - A.cta0[pq];
     const int S = A.splits[pq];
-    const int col0 = jb * A.nb, col1 = je * A.nb;       // needed columns (= B rows loaded)
     const int rcn = n2 / 8, rc0 = col0 / 8;             // rows of 8 r' per plane; first one loaded
-    const int nrow = (col1 - col0) / 8;                 // rows loaded per plane (a multiple of fbox)
+    const int nrow = cols / 8;                          // rows loaded per plane (a multiple of 16)
     const uint32_t plane_bytes = (uint32_t)nrow * 256u;
     // the row block's own 16 rows (the A operand before scaling by m): inside the loaded B
     // rows, or loaded separately into the A area of the stage
-    const bool own_in = !SEP || (16 * i >= rc0 && 16 * i + 16 <= rc0 + nrow);
+    const bool own_in = !SEP || 16 * i >= rc0;
     const uint32_t tx_bytes = 2u * plane_bytes + (own_in ? 0u : 2u * 16u * 256u);
+    const uint32_t st_bytes = ST_FB + 2u * plane_bytes;
+    const int nst = fwd_stages(cols);
     const int n_tiles = (G.npix + TP - 1) / TP;
     const int nsl_all = n_tiles * 8;
     const int cps = (nsl_all + S - 1) / S;
     const int sbeg = min(nsl_all, sp * cps), send = min(nsl_all, sbeg + cps);
     const int nq = send - sbeg;
     if (tid == 0) {
-        for (int k = 0; k < NST; ++k) {
-            tc::mbar_init(tc::smem_u32(&s_full_a[k]), NPROD_F / 32);
+        for (int k = 0; k < nst; ++k) {
+            tc::mbar_init(tc::smem_u32(&s_full_a[k]), 4);
             tc::mbar_init(tc::smem_u32(&s_full_b[k]), 1);
             tc::mbar_init(tc::smem_u32(&s_empty[k]), 1);
         }
@@ -937,152 +944,152 @@ __global__ void __launch_bounds__(NTHR_F, 1) k_forward_tc(FwdArgs A, const __gri
     tc::fence_before();
     __syncthreads();
     tc::fence_after();
-    const uint32_t tmem = s_tmem;
-    auto stage = [&](int k) { return smem + (size_t)k * ST_BYTES; };
+    const uint32_t tmem = __shfl_sync(0xffffffffu, s_tmem, 0);
+    const uint32_t smem0 = tc::smem_u32(smem), full_a0 = tc::smem_u32(&s_full_a[0]), full_b0 = tc::smem_u32(&s_full_b[0]);
+    const uint32_t empty0 = tc::smem_u32(&s_empty[0]);
 
     if (warp == NPROD_F / 32 + 1) {
         // ------------------------------ loader ------------------------------
-        if (lane == 0) {
-            int ql = 0;
-            bool err = false;
-            const uint64_t tm = reinterpret_cast<uint64_t>(&tmap);
-            const uint64_t tm16 = reinterpret_cast<uint64_t>(&tmap16);   // 16-row boxes: a row block's own rows
-            for (; ql < nq; ++ql) {
-                const int k = ql % NST;
-                if (ql >= NST && !tc::mbar_wait(tc::smem_u32(&s_empty[k]), (uint32_t)((ql / NST) - 1) & 1u, kMaxTries)) {
-                    err = true;
-                    break;
-                }
-                if (s_err) break;
-                const int sg = sbeg + ql, t = sg >> 3, x = (sg & 7) * 128;
-                const uint32_t mb = tc::smem_u32(&s_full_b[k]);
-                asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(mb), "r"(tx_bytes)
-                             : "memory");
+        const bool lead = tc::elect_one();
+        const uint64_t tm = reinterpret_cast<uint64_t>(&tmap);
+        const uint64_t tm16 = reinterpret_cast<uint64_t>(&tmap16);   // 16-row boxes
+        int ql = 0, k = 0;
+        uint32_t ph = 0;
+        bool ok = true;
+        for (; ql < nq; ++ql) {
+            if (ql >= nst && !tc::mbar_wait_warp(empty0 + 8u * k, ph ^ 1u, kMaxTries, &s_err)) {
+                ok = false;
+                break;
+            }
+            const int sg = sbeg + ql, x = (sg & 7) * 128, y0 = (sg >> 3) * 2 * rcn;
+            const uint32_t mb = full_b0 + 8u * k, st = smem0 + (uint32_t)k * st_bytes;
+            if (lead) {
+                tc::bulk_arm(mb, tx_bytes);
                 for (int hl = 0; hl < 2; ++hl) {
-                    for (int b = 0; b < nrow / A.fbox; ++b) {
-                        const uint32_t dst = tc::smem_u32(stage(k) + ST_FB + hl * plane_bytes + (uint32_t)(b * A.fbox) * 256u);
-                        const int y = (t * 2 + hl) * rcn + rc0 + b * A.fbox;
-                        asm volatile(
-                            "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
-                            ::"r"(dst), "l"(tm), "r"(x), "r"(y), "r"(mb)
-                            : "memory");
-                    }
-                    if (!own_in) {
-                        const uint32_t dst = tc::smem_u32(stage(k) + hl * ST_ALO);
-                        const int y = (t * 2 + hl) * rcn + 16 * i;
-                        asm volatile(
-                            "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
-                            ::"r"(dst), "l"(tm16), "r"(x), "r"(y), "r"(mb)
-                            : "memory");
-                    }
+                    const int y = y0 + hl * rcn;
+                    const uint32_t dst = st + ST_FB + (uint32_t)hl * plane_bytes;
+                    for (int b = 0; b < nrow; b += FBOX)
+                        tc::tma_2d(dst + (uint32_t)b * 256u, nrow - b >= FBOX ? tm : tm16, x, y + rc0 + b, mb);
+                    if (!own_in) tc::tma_2d(st + (uint32_t)hl * ST_ALO, tm16, x, y + 16 * i, mb);
                 }
             }
-            if (err || s_err) {
-                s_err = 1;
-                for (int x = (ql > NST ? ql - NST : 0); x < ql; ++x)
-                    tc::mbar_wait(tc::smem_u32(&s_full_b[x % NST]), (uint32_t)(x / NST) & 1u, kMaxTries);
-            }
+            if (++k == nst) { k = 0; ph ^= 1u; }
+        }
+        if (!ok && lead) {
+            s_err = 1;
+            for (int x = (ql > nst ? ql - nst : 0); x < ql; ++x)
+                tc::mbar_wait(full_b0 + 8u * (x % nst), (uint32_t)(x / nst) & 1u, kMaxTries);
         }
         __syncwarp();
     } else if (warp == NPROD_F / 32) {
         // ------------------------------ MMA issuer ------------------------------
-        if (lane == 0) {
-            // both operands MN-major (transpose bits 15 and 16): LBO = stride between the
-            // two 8-pixel K cores (128 B), SBO = stride between 8-r' cores (256 B)
-            const uint32_t id = tc::idesc_bf16_f32(128, (uint32_t)A.nb) | (1u << 15) | (1u << 16);
-            int last = -1;
-            bool err = false;
-            for (int q = 0; q < nq && !err; ++q) {
-                const int k = q % NST;
-                const uint32_t ph = (uint32_t)(q / NST) & 1u;
-                if (!tc::mbar_wait(tc::smem_u32(&s_full_a[k]), ph, kMaxTries)) { err = true; break; }
-                if (!tc::mbar_wait(tc::smem_u32(&s_full_b[k]), ph, kMaxTries)) { err = true; break; }
-                if (s_err) { err = true; break; }
-                tc::fence_after();
-                const uint32_t sa = tc::smem_u32(stage(k)), sb = sa + ST_FB;
-                const uint64_t dah = tc::sdesc(sa, 128, 256), dal = tc::sdesc(sa + ST_ALO, 128, 256);
-                for (int j = jb; j < je; ++j) {
-                    const uint32_t boff = (uint32_t)((j * A.nb) / 8 - rc0) * 256u;
-                    const uint64_t dbh = tc::sdesc(sb + boff, 128, 256);
-                    const uint64_t dbl = tc::sdesc(sb + plane_bytes + boff, 128, 256);
-                    const uint32_t d = tmem + (uint32_t)((j - jb) * A.nb);
-                    tc::mma_bf16(d, dah, dbh, id, q > 0 ? 1u : 0u);
-                    tc::mma_bf16(d, dah, dbl, id, 1u);
-                    tc::mma_bf16(d, dal, dbh, id, 1u);
+        // both operands MN-major (transpose bits 15 and 16): LBO = stride between the
+        // two 8-pixel K cores (128 B), SBO = stride between 8-r' cores (256 B)
+        const bool lead = tc::elect_one();
+        const uint32_t id0 = tc::idesc_bf16_f32(128, 0) | (1u << 15) | (1u << 16);
+        // one or two N-blocks: what exceeds 256 columns, then the last 256
+        const uint32_t n1 = cols > 256 ? (uint32_t)cols - 256u : (uint32_t)cols;
+        const uint32_t id1 = id0 | ((n1 >> 3) << 17), id2 = id0 | ((256u >> 3) << 17);
+        int k = 0, last = -1;
+        uint32_t ph = 0, last_ph = 0;
+        bool ok = true;
+        for (int q = 0; q < nq; ++q) {
+            ok = tc::mbar_wait_warp(full_b0 + 8u * k, ph, kMaxTries, &s_err) &&
+                 tc::mbar_wait_warp(full_a0 + 8u * k, ph, kMaxTries, &s_err);
+            if (!ok) break;
+            tc::fence_after();
+            const uint32_t sa = smem0 + (uint32_t)k * st_bytes, sb = sa + ST_FB;
+            const uint64_t dah = tc::sdesc(sa, 128, 256), dal = tc::sdesc(sa + ST_ALO, 128, 256);
+            const uint64_t dbh = tc::sdesc(sb, 128, 256), dbl = tc::sdesc(sb + plane_bytes, 128, 256);
+            const uint32_t acc = q > 0 ? 1u : 0u;
+            if (lead) {
+                tc::mma_bf16(tmem, dah, dbh, id1, acc);
+                tc::mma_bf16(tmem, dah, dbl, id1, 1u);
+                tc::mma_bf16(tmem, dal, dbh, id1, 1u);
+                if (cols > 256) {
+                    const uint64_t dbh2 = dbh + 2u * n1, dbl2 = dbl + 2u * n1;   // 32 bytes a column
+                    tc::mma_bf16(tmem + n1, dah, dbh2, id2, acc);
+                    tc::mma_bf16(tmem + n1, dah, dbl2, id2, 1u);
+                    tc::mma_bf16(tmem + n1, dal, dbh2, id2, 1u);
                 }
-                tc::commit(tc::smem_u32(&s_empty[k]));
+                tc::commit(empty0 + 8u * k);
                 if (q == nq - 1) tc::commit(tc::smem_u32(&s_acc_full));
-                last = q;
             }
-            if (err) {
-                s_err = 1;
-                atomicAdd(A.counters + CNT_TC_TIMEOUT, 1u);
-                if (last >= 0) tc::mbar_wait(tc::smem_u32(&s_empty[last % NST]), (uint32_t)(last / NST) & 1u, kMaxTries);
-            }
+            last = k;
+            last_ph = ph;
+            if (++k == nst) { k = 0; ph ^= 1u; }
+        }
+        if (!ok && lead) {
+            s_err = 1;
+            atomicAdd(A.counters + CNT_TC_TIMEOUT, 1u);
+            if (last >= 0) tc::mbar_wait(empty0 + 8u * last, last_ph, kMaxTries);   // the MMAs still in flight
         }
         __syncwarp();
     } else {
         // -------------------------------- producers --------------------------------
-        // thread tid: row rl = tid / 16 of 8 r' (of the row block's 16), K core pc = (tid / 8) % 2,
-        // pixel row x8 = tid % 8 of that core
-        const int rl = tid >> 4, pc = (tid >> 3) & 1, x8 = tid & 7;
+        // thread u of its group of 128: K core pc = (u / 8) % 2, pixel row x8 = u % 8 of that core,
+        // rows rl = u / 16 and rl + 8 of 8 r' (of the row block's 16)
+        constexpr int NG = 4;
+        const int grp = warp >> 2, u = tid & 127;
+        const int rl = u >> 4, pc = (u >> 3) & 1, x8 = u & 7;
         const uint32_t aoff = (uint32_t)(rl * 256 + pc * 128 + x8 * 16);
         // source of this thread's 16 bytes: the B rows, or the A area itself (scaled in place)
         const uint32_t soff = own_in ? ST_FB + (uint32_t)((16 * i - rc0 + rl) * 256 + pc * 128 + x8 * 16) : aoff;
         const uint32_t slo = own_in ? plane_bytes : ST_ALO;
-        bool err = false;
+        bool ok = true;
         auto load_m = [&](int q) -> float {
             if (q >= nq) return 0.f;
             const int px = (sbeg + q) * 16 + pc * 8 + x8;
             return px < G.npix ? __ldg(A.m + px) : 0.f;
         };
-        float mnext = load_m(0);
-        for (int q = 0; q < nq; ++q) {
-            const int k = q % NST;
-            const uint32_t ph = (uint32_t)(q / NST) & 1u;
+        float mnext = load_m(grp);
+        int k = grp % nst;   // nst >= NG + 1
+        uint32_t ph = 0;
+        for (int q = grp; q < nq; q += NG) {
             const float mm = mnext;
-            mnext = load_m(q + 1);
-            if (!err && q >= NST) err = !tc::mbar_wait(tc::smem_u32(&s_empty[k]), ph ^ 1u, kMaxTries);
-            if (!err) err = !tc::mbar_wait(tc::smem_u32(&s_full_b[k]), ph, kMaxTries);
-            err = __any_sync(0xffffffffu, err || s_err != 0);
-            if (!err) {
-                const unsigned char* src = stage(k) + soff;
+            mnext = load_m(q + NG);
+            // The stage's previous slice, another group's, has been used: without this wait the
+            // test of the full barrier below could see the phase before it.  (This test cannot:
+            // this group's last slice q - NG had landed, so its loader had seen slices up to
+            // q - NG - nst, among them the stage's last but one, q - 2 nst, used.)
+            if (q >= nst) ok = ok && tc::mbar_wait_warp(empty0 + 8u * k, ph ^ 1u, kMaxTries, &s_err);
+            ok = ok && tc::mbar_wait_warp(full_b0 + 8u * k, ph, kMaxTries, &s_err);
+            if (!ok) break;
+            unsigned char* st = smem + (size_t)k * st_bytes;
+#pragma unroll
+            for (int x = 0; x < 2; ++x) {
+                const unsigned char* src = st + soff + 2048u * x;
                 const uint4 vh = *(const uint4*)src, vl = *(const uint4*)(src + slo);
                 const uint32_t hw[4] = {vh.x, vh.y, vh.z, vh.w}, lw[4] = {vl.x, vl.y, vl.z, vl.w};
                 uint32_t oh[4], ol[4];
 #pragma unroll
                 for (int t = 0; t < 4; ++t) {
-                    const float x0 = (__bfloat162float(__ushort_as_bfloat16((unsigned short)(hw[t] & 0xffff))) +
-                                      __bfloat162float(__ushort_as_bfloat16((unsigned short)(lw[t] & 0xffff)))) * mm;
-                    const float x1 = (__bfloat162float(__ushort_as_bfloat16((unsigned short)(hw[t] >> 16))) +
-                                      __bfloat162float(__ushort_as_bfloat16((unsigned short)(lw[t] >> 16)))) * mm;
                     __nv_bfloat16 h0, l0, h1, l1;
-                    tc::split_bf16(x0, h0, l0);
-                    tc::split_bf16(x1, h1, l1);
+                    tc::split_bf16(sum_lo16(hw[t], lw[t]) * mm, h0, l0);
+                    tc::split_bf16(sum_hi16(hw[t], lw[t]) * mm, h1, l1);
                     oh[t] = pack2(h0, h1);
                     ol[t] = pack2(l0, l1);
                 }
-                *(uint4*)(stage(k) + aoff) = make_uint4(oh[0], oh[1], oh[2], oh[3]);
-                *(uint4*)(stage(k) + ST_ALO + aoff) = make_uint4(ol[0], ol[1], ol[2], ol[3]);
+                *(uint4*)(st + aoff + 2048u * x) = make_uint4(oh[0], oh[1], oh[2], oh[3]);
+                *(uint4*)(st + ST_ALO + aoff + 2048u * x) = make_uint4(ol[0], ol[1], ol[2], ol[3]);
             }
             tc::fence_proxy_async();
             __syncwarp();
-            if (lane == 0 && !err) tc::mbar_arrive(tc::smem_u32(&s_full_a[k]));
+            if (lane == 0) tc::mbar_arrive(full_a0 + 8u * k);
+            k += NG;
+            if (k >= nst) { k -= nst; ph ^= 1u; }
         }
         // epilogue: this CTA's partial D block (128 rows x needed columns) to global memory
-        if (!err && nq > 0) err = !tc::mbar_wait(tc::smem_u32(&s_acc_full), 0u, kMaxTries);
-        err = __any_sync(0xffffffffu, err || s_err != 0);
+        if (nq > 0) ok = ok && tc::mbar_wait_warp(tc::smem_u32(&s_acc_full), 0u, kMaxTries, &s_err);
         tc::fence_after();
-        if (!err) {
-            const int row = tid & 127, g = tid >> 7;
+        if (ok) {
+            const int row = tid & 127, g = warp >> 2;
             const uint32_t lane_off = (uint32_t)((warp & 3) * 32) << 16;
-            float* out = A.partial + ((size_t)blockIdx.x * 128 + row) * n2;
-            int cnum = 0;
-            for (int cb = col0; cb < col1; cb += 32, ++cnum) {
-                if ((cnum & 1) != g) continue;
+            float* out = A.partial + ((size_t)blockIdx.x * 128 + row) * n2 + col0;
+            for (int cb = 32 * g; cb < cols; cb += 128) {
                 float v[32];
                 if (nq > 0) {
-                    tc::tmem_ld32(tmem + lane_off + (uint32_t)(cb - col0), v);
+                    tc::tmem_ld32(tmem + lane_off + (uint32_t)cb, v);
                 } else {
 #pragma unroll
                     for (int t = 0; t < 32; ++t) v[t] = 0.f;
@@ -1090,6 +1097,8 @@ __global__ void __launch_bounds__(NTHR_F, 1) k_forward_tc(FwdArgs A, const __gri
 #pragma unroll
                 for (int t = 0; t < 32; t += 4) *(float4*)(out + cb + t) = make_float4(v[t], v[t + 1], v[t + 2], v[t + 3]);
             }
+        } else {
+            s_err = 1;
         }
     }
     tc::fence_before();
@@ -1097,108 +1106,144 @@ __global__ void __launch_bounds__(NTHR_F, 1) k_forward_tc(FwdArgs A, const __gri
     if (warp == 0) tc::tmem_dealloc(tmem, A.tmem_cols);
 }
 
-// d = w^2 (sum over splits of the partial D blocks, symmetric lookup), and
-// per-block partial sums of W |d|^2.
 // d = w^2 (sum over splits of the partial D blocks), and per-block partial sums of
 // W |d|^2.  D and d are symmetric, and for e <= r the 2 x 2 block of D at (2e, 2r) lies in
-// a computed block (on or above the block diagonal), so thread (e, r), e <= r, reads it
-// row-wise (consecutive threads, consecutive r: coalesced) and writes d[e][r] and d[r][e].
-__global__ void k_forward_tc_reduce(FwdArgs A, float2* __restrict__ d_out, const uint8_t* __restrict__ w,
-                                    double* __restrict__ den_part) {
-    const int n = A.G.n_elem, n2 = 2 * n;
+// a computed block (right of its row block's first column), so entry (e, r), e <= r, is
+// read row-wise and written to d[e][r] and d[r][e].  YS warps take 32 consecutive r of one e:
+// each every YS-th split, the first adds the warps' sums in order.  YS = 1 where the
+// entries alone fill the chip (256 elements: 12 us for 52 splits; eight warps an entry, with
+// their barriers, 43), 8 below 128 elements (64: 27 us by single warps, 152 splits each).
+template <int YS>
+__global__ void __launch_bounds__(256) k_forward_tc_reduce(FwdArgs A, float2* __restrict__ d_out, const uint8_t* __restrict__ w,
+                                                           double* __restrict__ den_part) {
+    __shared__ float4 s_sum[8][32];
+    __shared__ double s_den[8];
+    const int n = A.G.n_elem, n2 = 2 * n, lane = threadIdx.x & 31, wid = threadIdx.x >> 5, y = wid % YS;
     double acc = 0.0;
-    const long long total = (long long)n * n;
-    for (long long jj = blockIdx.x * (long long)blockDim.x + threadIdx.x; jj < total;
-         jj += (long long)gridDim.x * blockDim.x) {
-        const int e = (int)(jj / n), r = (int)(jj % n);
-        if (e > r) continue;
-        const int i = (2 * e) >> 7, row = (2 * e) & 127;
-        const int pq = A.pidx[i][((2 * r) / A.nb) >> 1];
-        float2 d0 = make_float2(0.f, 0.f), d1 = make_float2(0.f, 0.f);   // D[2e][2r..2r+1], D[2e+1][2r..2r+1]
-        for (int sp = 0; sp < A.splits[pq]; ++sp) {
-            const float* blk = A.partial + ((size_t)(A.cta0[pq] + sp) * 128 + row) * n2 + 2 * r;
-            const float2 a0 = *(const float2*)blk, a1 = *(const float2*)(blk + n2);
-            d0.x += a0.x;
-            d0.y += a0.y;
-            d1.x += a1.x;
-            d1.y += a1.y;
+    const int nrb = n / 32;   // n is a multiple of 64
+    constexpr int TPB = 8 / YS;   // runs of 32 entries a CTA takes at a time
+    for (int run0 = blockIdx.x * TPB; run0 < n * nrb; run0 += gridDim.x * TPB) {
+        const int run = run0 + wid / YS;   // n nrb is a multiple of 8
+        const int e = run / nrb, r = 32 * (run - e * nrb) + lane;
+        const bool live = e <= r;
+        float4 s = make_float4(0.f, 0.f, 0.f, 0.f);   // D[2e][2r..2r+1], D[2e+1][2r..2r+1]
+        if (live) {
+            const int i = (2 * e) >> 7, row = (2 * e) & 127, pq = A.pidx[i][(2 * r) >> 9], ns = A.splits[pq];
+            const float* blk = A.partial + ((size_t)A.cta0[pq] * 128 + row) * n2 + 2 * r;
+            const size_t step = (size_t)128 * n2;
+#pragma unroll 8
+            for (int sp = y; sp < ns; sp += YS) {
+                const float2 a0 = *(const float2*)(blk + sp * step), a1 = *(const float2*)(blk + sp * step + n2);
+                s.x += a0.x;
+                s.y += a0.y;
+                s.z += a1.x;
+                s.w += a1.y;
+            }
         }
-        // the image rows 2r + 1 hold -Im G_r (the conjugate, as the adjoint uses it), so the
-        // product of the two images is conj(d): Re d as is, Im d negated
-        const float dre = (d0.x - d1.y) * A.F.w2;
-        const float dim = -(d0.y + d1.x) * A.F.w2;
-        const size_t er = (size_t)e * n + r, re = (size_t)r * n + e;
-        if (d_out) {
-            d_out[er] = make_float2(dre, dim);
-            if (e != r) d_out[re] = make_float2(dre, dim);
+        if (YS > 1) {
+            __syncthreads();
+            s_sum[wid][lane] = s;
+            __syncthreads();
+            if (y == 0)
+                for (int k = 1; k < YS; ++k) {
+                    const float4 o = s_sum[wid + k][lane];
+                    s.x += o.x;
+                    s.y += o.y;
+                    s.z += o.z;
+                    s.w += o.w;
+                }
         }
-        if (w) {
-            const int cnt = (w[er] ? 1 : 0) + ((e != r && w[re]) ? 1 : 0);
-            if (cnt) acc += cnt * ((double)dre * dre + (double)dim * dim);
+        if (y == 0 && live) {
+            // the image rows 2r + 1 hold -Im G_r (the conjugate, as the adjoint uses it), so the
+            // product of the two images is conj(d): Re d as is, Im d negated
+            const float dre = (s.x - s.w) * A.w2;
+            const float dim = -(s.y + s.z) * A.w2;
+            const size_t er = (size_t)e * n + r, re = (size_t)r * n + e;
+            if (d_out) {
+                d_out[er] = make_float2(dre, dim);
+                if (e != r) d_out[re] = make_float2(dre, dim);
+            }
+            if (w) {
+                const int cnt = (w[er] ? 1 : 0) + ((e != r && w[re]) ? 1 : 0);
+                if (cnt) acc += cnt * ((double)dre * dre + (double)dim * dim);
+            }
         }
     }
     if (den_part) {
-        __shared__ double sred[256];
-        sred[threadIdx.x] = acc;
+        for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
+        if (lane == 0) s_den[wid] = acc;
         __syncthreads();
-        for (int k = blockDim.x / 2; k > 0; k >>= 1) {
-            if (threadIdx.x < k) sred[threadIdx.x] += sred[threadIdx.x + k];
-            __syncthreads();
+        if (threadIdx.x == 0) {
+            for (int k = 1; k < 8; ++k) acc += s_den[k];
+            den_part[blockIdx.x] = acc;
         }
-        if (threadIdx.x == 0) den_part[blockIdx.x] = sred[0];
     }
+}
+
+cudaError_t forward_tc_reduce(const FwdArgs& A, float2* d_out, const uint8_t* w, double* den_part, cudaStream_t s) {
+    if (A.G.n_elem < 128) k_forward_tc_reduce<8><<<256, 256, 0, s>>>(A, d_out, w, den_part);
+    else k_forward_tc_reduce<1><<<256, 256, 0, s>>>(A, d_out, w, den_part);
+    return cudaGetLastError();
 }
 
 FwdArgs make_fwd_args(const GeoDev& G, const FreqC& F, const float* m, float* partial, int n_ctas,
                       uint32_t* counters) {
     FwdArgs A;
     A.G = G;
-    A.F = F;
+    A.w2 = F.w2;
     A.m = m;
     A.partial = partial;
     A.counters = counters;
     const int n2 = 2 * G.n_elem;
     A.n_mb = n2 / 128;
-    A.nbn = (n2 + 255) / 256;
-    A.nb = n2 / A.nbn;
-    // pairs (row block i, column blocks [jb, je)): blocks from the diagonal one on, in
-    // groups of two (group g holds blocks 2g and 2g + 1)
+    // pairs (row block i, columns from its diagonal on), in groups of 512 columns
     A.n_pairs = 0;
+    int widest = 0;
+    double cost[FMAXP], total = 0.0;
     for (int i = 0; i < A.n_mb; ++i) {
         for (int g = 0; g < FMAXG; ++g) A.pidx[i][g] = -1;
-        const int jmin = jmin_of(i, A.nb);
-        for (int g = jmin / 2; 2 * g < A.nbn; ++g) {
+        for (int g = (128 * i) / 512; 512 * g < n2; ++g) {
             const int q = A.n_pairs++;
             A.p_i[q] = i;
-            A.p_jb[q] = 2 * g > jmin ? 2 * g : jmin;
-            A.p_je[q] = 2 * g + 2 < A.nbn ? 2 * g + 2 : A.nbn;
+            A.p_c0[q] = 128 * i > 512 * g ? 128 * i : 512 * g;
+            A.p_c1[q] = 512 * (g + 1) < n2 ? 512 * (g + 1) : n2;
             A.pidx[i][g] = q;
+            const int cols = A.p_c1[q] - A.p_c0[q];
+            if (cols > widest) widest = cols;
+            // A slice's cost in KB of shared-memory traffic, which sets the pace of the wide pairs:
+            // the operands' arrival, the producers' 16 KB, and per N-block three MMAs reading A
+            // (4 KB) and their columns of B; never below what a slice takes by latency alone.
+            // Forward stage of four frequencies, 256 elements at 512 x 512 pixels, by that floor:
+            // 60 KB 834 us, 80 KB 819, 100 KB 876, all pairs alike 940
+            const double kb = cols / 16.0 + 16.0 + 12.0 * (cols > 256 ? 2 : 1) + 0.09375 * cols;
+            cost[q] = kb > FWD_MIN_KB ? kb : FWD_MIN_KB;
+            total += cost[q];
         }
     }
-    // TMEM: the widest pair, two blocks (one when there is only one)
-    uint32_t cols = 32;
-    while (cols < (uint32_t)((A.nbn > 1 ? 2 : 1) * A.nb)) cols <<= 1;
-    A.tmem_cols = cols;
-    // splits per pair: equal.  A pixel slice costs about the same on every pair, whether
-    // it issues MMAs for one column block or two (the operand delivery and producer work
-    // per slice, not the tensor pipe, set the pace), so splits in proportion to the
-    // column blocks left the pairs with one block idle half the time.
+    A.tmem_cols = 32;
+    while (A.tmem_cols < (uint32_t)widest) A.tmem_cols <<= 1;
+    // splits in proportion to that cost, every pair at least one, no split below 8 slices
+    const int nsl = ((G.npix + TP - 1) / TP) * 8;
+    const int most = nsl / 8 > 0 ? nsl / 8 : 1;
+    int left = n_ctas;
+    for (int q = 0; q < A.n_pairs; ++q) {
+        A.splits[q] = (int)(n_ctas * cost[q] / total);
+        if (A.splits[q] < 1) A.splits[q] = 1;
+        left -= A.splits[q];
+    }
+    while (left-- > 0) {   // what rounding left over goes to the slowest pair
+        int slow = 0;
+        for (int q = 1; q < A.n_pairs; ++q)
+            if (cost[q] / A.splits[q] > cost[slow] / A.splits[slow]) slow = q;
+        ++A.splits[slow];
+    }
     int c0 = 0;
     for (int q = 0; q < A.n_pairs; ++q) {
-        int sq = n_ctas / A.n_pairs;
-        if (sq < 1) sq = 1;
-        A.splits[q] = sq;
+        if (A.splits[q] > most) A.splits[q] = most;
         A.cta0[q] = c0;
-        c0 += sq;
+        c0 += A.splits[q];
     }
     A.cta0[A.n_pairs] = c0;
-    // TMA box height of the B rows: the largest power of two up to FBOX_MAX dividing every
-    // pair's loaded rows (a row block's own 16 rows, where loaded apart, use 16-row boxes)
-    A.fbox = FBOX_MAX;
-    for (int q = 0; q < A.n_pairs; ++q) {
-        const int nrow = (A.p_je[q] - A.p_jb[q]) * A.nb / 8;
-        while (nrow % A.fbox != 0) A.fbox >>= 1;
-    }
     return A;
 }
 
@@ -1216,19 +1261,15 @@ cudaError_t forward_tc_kernel(const GeoDev& G, const void* aimg, const FreqC& F,
     if (!tc_adjoint_supported(G.n_elem) || !aimg) return cudaErrorInvalidValue;
     const FwdArgs A = make_fwd_args(G, F, m, partial, n_ctas, counters);
     // the A image of this frequency as a 2-D tensor: rows of 8 r' x 128 pixels (1024 bf16),
-    // (tile, plane, row) major; boxes of 128 elements (one 16-pixel slice) x fbox rows
+    // (tile, plane, row) major; boxes of 128 elements (one 16-pixel slice) x 32 or 16 rows
     const int rcn = 2 * G.n_elem / 8;
     const int n_tiles = (G.npix + TP - 1) / TP;
     CUtensorMap tmap, tmap16;
-    if (A.fbox < 1 || !tc::encode_tmap_2d(&tmap, aimg, 1024, (uint64_t)n_tiles * 2 * rcn, 2048, 128, (uint32_t)A.fbox))
+    if (!tc::encode_tmap_2d(&tmap, aimg, 1024, (uint64_t)n_tiles * 2 * rcn, 2048, 128, (uint32_t)FBOX) ||
+        !tc::encode_tmap_2d(&tmap16, aimg, 1024, (uint64_t)n_tiles * 2 * rcn, 2048, 128, 16u))
         return cudaErrorUnknown;
-    if (!tc::encode_tmap_2d(&tmap16, aimg, 1024, (uint64_t)n_tiles * 2 * rcn, 2048, 128, 16u)) return cudaErrorUnknown;
     const int sm = NST * (int)ST_BYTES;
-    bool sep = false;
-    for (int q = 0; q < A.n_pairs; ++q) {
-        const int rc0 = A.p_jb[q] * A.nb / 8, nrow = (A.p_je[q] - A.p_jb[q]) * A.nb / 8;
-        sep = sep || !(16 * A.p_i[q] >= rc0 && 16 * A.p_i[q] + 16 <= rc0 + nrow);
-    }
+    const bool sep = G.n_elem > 256;   // a column group left of which a row block lies
     cudaError_t e;
     if (sep) {
         e = cudaFuncSetAttribute(k_forward_tc<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
@@ -1251,8 +1292,7 @@ cudaError_t launch_forward_tc(const GeoDev& G, const void* aimg, const FreqC& F,
     FwdArgs A;
     cudaError_t e = forward_tc_kernel(G, aimg, F, m, partial, n_ctas, counters, s, &A);
     if (e != cudaSuccess) return e;
-    k_forward_tc_reduce<<<256, 256, 0, s>>>(A, d_out, w, den_part);
-    return cudaGetLastError();
+    return forward_tc_reduce(A, d_out, w, den_part, s);
 }
 
 cudaError_t launch_forward_tc_overlap(const GeoDev& G, const void* aimg, const FreqC& F, const float* m,
@@ -1264,7 +1304,6 @@ cudaError_t launch_forward_tc_overlap(const GeoDev& G, const void* aimg, const F
     if (e == cudaSuccess) e = cudaEventRecord(fwd_done, s);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(r, fwd_done, 0);
     if (e != cudaSuccess) return e;
-    k_forward_tc_reduce<<<256, 256, 0, r>>>(A, d_out, w, den_part);
-    e = cudaGetLastError();
+    e = forward_tc_reduce(A, d_out, w, den_part, r);
     return e == cudaSuccess ? cudaEventRecord(red_done, r) : e;
 }

@@ -189,6 +189,14 @@ __device__ __forceinline__ void bulk_copy_hint(uint32_t dst, const void* src, ui
                  : "memory");
 }
 
+// One thread: a 2-D tiled TMA load of the tensor map's box at (x, y) (x * element size a
+// multiple of 16 bytes) that completes its bytes on the armed barrier.
+__device__ __forceinline__ void tma_2d(uint32_t dst, uint64_t tmap, int x, int y, uint32_t mbar) {
+    asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
+                 ::"r"(dst), "l"(tmap), "r"(x), "r"(y), "r"(mbar)
+                 : "memory");
+}
+
 // TMEM allocation by one full warp; the base address is written to *slot (shared).
 __device__ __forceinline__ void tmem_alloc(uint32_t slot_saddr, uint32_t ncols) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(slot_saddr), "r"(ncols)
