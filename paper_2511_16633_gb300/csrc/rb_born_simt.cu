@@ -78,8 +78,9 @@ __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
 // Chunks of 32 r x 32 e (16 KB) go through two shared-memory buffers (cp.async); of each
 // chunk, the CTA's four groups of 64 threads take 8 r each, and a thread accumulates 4
 // elements x 4 pixels of U and V over its group's r.  g and H are linear in U and V, so the
-// groups' parts meet only in the final sums.  Bound by the FP32 pipe: 88 FMAs per 6
-// shared-memory loads.
+// groups' parts meet only in the final sums.  Bound by the FP32 pipe and issue: 88 FMAs per 6
+// shared-memory loads.  100 elements, 251 x 237 pixels: 370 -> 219 us; 150 elements, 260 x
+// 243, two frequencies: 2553 -> 637 us (the full sums, rows of T loaded one by one).
 __global__ void __launch_bounds__(AT, 2) k_adjoint_simt(GeoDev G, const rb_cell* __restrict__ tables, const float* __restrict__ c,
                                                         FreqSet F, const float4* __restrict__ sym, float2* __restrict__ g_out,
                                                         float* __restrict__ h_out, float* __restrict__ gsum,
@@ -209,8 +210,9 @@ constexpr int FTHR = 128;   // 8 x 16 threads, 8 x 4 complex outputs each
 
 // FROM_G: G of the frequency comes from the buffer g [n_elem][npix]; otherwise (no workspace)
 // it is synthesised from the tables, once per tile pair that uses it.  Bound by the FP32
-// pipe: 128 FMAs per pixel and thread for 6 shared-memory loads (a 4 x 4 tile and G
-// synthesised for every pair: half the time was the synthesis).
+// pipe: 128 FMAs per pixel and thread for 6 shared-memory loads.  150 elements, 260 x 243
+// pixels: 416 us and 72 for G (1189 us with a 4 x 4 tile a thread and G synthesised for every
+// pair, half the time the synthesis).
 template <bool FROM_G>
 __global__ void __launch_bounds__(FTHR) k_forward_simt(GeoDev G, const float2* __restrict__ g, const rb_cell* __restrict__ tables,
                                                        const float* __restrict__ c, FreqC F, const float* __restrict__ m,
