@@ -48,18 +48,28 @@ struct Deriv { float x, y, th, t, q, p, l; };
 // record holds per field the coefficients (a, b, c, d) of a + b u + c v + d u v over the
 // cell's unit square, paired fields side by side (rb_fields.cu), so each pair takes three
 // packed two-lane FMAs (same operations and rounding as three scalar ones per field).
-// The cell indices stay floats (floorf), and the record is reloaded only when the ray
-// changes cell.
+// The cell indices stay floats (floorf), and the record is reloaded only by the lanes whose
+// ray changes cell.  The lanes' records are on lines of their own, so each load costs the
+// LSU a wavefront per lane whatever its width: four 32-byte loads instead of seven of 16.
+// INSIDE: the query lies inside the grid (the launcher's rule: the ring plus a step does), so
+// it needs no clamping; the record's address is clamped all the same.
+template <bool INSIDE>
 __device__ __forceinline__ void sample(const GeoDev& G, const float4* __restrict__ cells, Cache& cc, float px, float py,
                                        float f[7]) {
-    const float u = fminf(fmaxf(fmaf(px, G.inv_h, G.cxg), 0.f), G.fxmax);
-    const float v = fminf(fmaxf(fmaf(py, G.inv_h, G.cyg), 0.f), G.fymax);
-    const float fi = fminf(floorf(u), G.fxmax - 1.f), fj = fminf(floorf(v), G.fymax - 1.f);
+    float u = fmaf(px, G.inv_h, G.cxg), v = fmaf(py, G.inv_h, G.cyg);
+    if (!INSIDE) {
+        u = fminf(fmaxf(u, 0.f), G.fxmax);
+        v = fminf(fmaxf(v, 0.f), G.fymax);
+    }
+    float fi = floorf(u), fj = floorf(v);
+    if (!INSIDE) {
+        fi = fminf(fi, G.fxmax - 1.f);
+        fj = fminf(fj, G.fymax - 1.f);
+    }
     const float fu = u - fi, fv = v - fj;
     if (fi != cc.fi || fj != cc.fj) {
-        // the lanes' records are on lines of their own, so each load costs the LSU a wavefront
-        // per lane whatever its width: four 32-byte loads instead of seven of 16 bytes
-        const float4* p = cells + ((size_t)(int)fj * (size_t)(G.nx - 1) + (size_t)(int)fi) * 8;
+        const int ci = min(max((int)fi, 0), G.nx - 2), cj = min(max((int)fj, 0), G.ny - 2);
+        const float4* p = cells + ((size_t)cj * (size_t)(G.nx - 1) + (size_t)ci) * 8;
         float4 pad;
         ldg32(p, cc.r[0], cc.r[1]);
         ldg32(p + 2, cc.r[2], cc.r[3]);
@@ -115,19 +125,17 @@ __device__ __forceinline__ void ray_sincos(float x, float* s, float* c) {
 
 // cos/sin of (th_hi + d) from cos/sin of th_hi and a small d (Taylor to d^7).
 __device__ __forceinline__ void rotate(float C0, float S0, float th_hi, float d, float& c, float& s) {
-    if (fabsf(d) < 0.2f) {
-        const float d2 = d * d;
-        const float cd = 1.f - 0.5f * d2 * (1.f - d2 * (1.f / 12.f) * (1.f - d2 * (1.f / 30.f)));
-        const float sd = d * (1.f - d2 * (1.f / 6.f) * (1.f - d2 * (1.f / 20.f) * (1.f - d2 * (1.f / 42.f))));
-        c = C0 * cd - S0 * sd;
-        s = S0 * cd + C0 * sd;
-    } else {
-        // a turn of 0.2 rad within half a step (gradients far beyond tissue): the hardware
-        // approximation (~1e-6 absolute), small enough not to weigh on the common path
-        __sincosf(th_hi + d, &s, &c);
-    }
+    const float d2 = d * d;
+    const float cd = 1.f - 0.5f * d2 * (1.f - d2 * (1.f / 12.f) * (1.f - d2 * (1.f / 30.f)));
+    const float sd = d * (1.f - d2 * (1.f / 6.f) * (1.f - d2 * (1.f / 20.f) * (1.f - d2 * (1.f / 42.f))));
+    c = C0 * cd - S0 * sd;
+    s = S0 * cd + C0 * sd;
+    // a turn of 0.2 rad within half a step (gradients far beyond tissue): the hardware
+    // approximation (~1e-6 absolute), small enough not to weigh on the common path
+    if (!(fabsf(d) < 0.2f)) __sincosf(th_hi + d, &s, &c);
 }
 
+template <bool INSIDE>
 __device__ __forceinline__ Deriv eval_stage(const GeoDev& G, const float4* __restrict__ cells, Cache& cc,
                                             float xh, float xl, float yh, float yl, float Ca, float Sa, float tha,
                                             float dth, float q, float p,
@@ -138,7 +146,7 @@ __device__ __forceinline__ Deriv eval_stage(const GeoDev& G, const float4* __res
     rotate(Ca, Sa, tha, fmaf(a, kp.th, dth), cth, sth);
     const float qs = fmaf(a, kp.q, q), ps = fmaf(a, kp.p, p);
     float f[7];
-    sample(G, cells, cc, px, py, f);
+    sample<INSIDE>(G, cells, cc, px, py, f);
     const float c = f[0];
     const float rc = __fdividef(1.0f, c);   // ~2 ulp: far below the RK4 truncation error
     Deriv d;
@@ -151,6 +159,27 @@ __device__ __forceinline__ Deriv eval_stage(const GeoDev& G, const float4* __res
     d.p = -(cnn * rc * rc) * qs;
     d.l = f[6];
     return d;
+}
+
+// RK4 increments of (x, y, th, T, Q, P, L) over one step.
+template <bool INSIDE>
+__device__ __forceinline__ Deriv rk4_step(const GeoDev& G, const float4* __restrict__ cells, Cache& cc, float xh, float xl, float yh,
+                                          float yl, float Ca, float Sa, float tha, float dth, float q, float p) {
+    const float ds = G.ds, a2 = 0.5f * G.ds, ds6 = G.ds * (1.0f / 6.0f);
+    const Deriv z{0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    const Deriv k1 = eval_stage<INSIDE>(G, cells, cc, xh, xl, yh, yl, Ca, Sa, tha, dth, q, p, 0.f, z);
+    const Deriv k2 = eval_stage<INSIDE>(G, cells, cc, xh, xl, yh, yl, Ca, Sa, tha, dth, q, p, a2, k1);
+    const Deriv k3 = eval_stage<INSIDE>(G, cells, cc, xh, xl, yh, yl, Ca, Sa, tha, dth, q, p, a2, k2);
+    const Deriv k4 = eval_stage<INSIDE>(G, cells, cc, xh, xl, yh, yl, Ca, Sa, tha, dth, q, p, ds, k3);
+    Deriv inc;
+    inc.x = ds6 * (k1.x + 2.f * k2.x + 2.f * k3.x + k4.x);
+    inc.y = ds6 * (k1.y + 2.f * k2.y + 2.f * k3.y + k4.y);
+    inc.th = ds6 * (k1.th + 2.f * k2.th + 2.f * k3.th + k4.th);
+    inc.t = ds6 * (k1.t + 2.f * k2.t + 2.f * k3.t + k4.t);
+    inc.q = ds6 * (k1.q + 2.f * k2.q + 2.f * k3.q + k4.q);
+    inc.p = ds6 * (k1.p + 2.f * k2.p + 2.f * k3.p + k4.p);
+    inc.l = ds6 * (k1.l + 2.f * k2.l + 2.f * k3.l + k4.l);
+    return inc;
 }
 
 __device__ __forceinline__ void comp_add(float& hi, float& lo, float inc) {
@@ -170,10 +199,12 @@ __device__ __noinline__ bool outside_ring(float xh, float xl, float yh, float yl
 
 __device__ __forceinline__ double exit_lambda(double ax, double ay, double bx, double by, double R) {
     const double dx = bx - ax, dy = by - ay;
-    const double qa = dx * dx + dy * dy;
-    const double qb = 2.0 * (ax * dx + ay * dy);
-    const double qc = ax * ax + ay * ay - R * R;
-    double disc = qb * qb - 4.0 * qa * qc;
+    // fused multiply-adds written out, so that every instance of the tracer forms the same bits
+    // (left to the compiler, they are paired differently from one instance to the next)
+    const double qa = __fma_rn(dy, dy, __dmul_rn(dx, dx));
+    const double qb = __dmul_rn(2.0, __fma_rn(ay, dy, __dmul_rn(ax, dx)));
+    const double qc = __fma_rn(-R, R, __fma_rn(ax, ax, __dmul_rn(ay, ay)));
+    double disc = __fma_rn(qb, qb, -__dmul_rn(__dmul_rn(4.0, qa), qc));
     if (disc < 0.0) disc = 0.0;
     const double sq = sqrt(disc);
     double lam;
@@ -320,11 +351,18 @@ __device__ __forceinline__ void put_vtx(Vtx* dst, const Vtx& v) {
     stg32(dst, make_float4(v.xh, v.xl, v.yh, v.yl), make_float4(v.t, v.q, v.l, __int_as_float(v.k)));
 }
 
-// One thread per ray: RK4 from the element to the ring, the end record, and (when
-// verts is set) every vertex into the vertex stream for the rasteriser.
+// One thread per ray: RK4 from the element to the ring, the end record, and (PUT) every
+// vertex into the vertex stream for the rasteriser, (SAMPLES) the caller's vertex arrays.
+// What bounds it is the length of a step's chain of dependent instructions (about 600, and
+// 3000 cycles even alone on an SM) times the steps of the longest rays; 13 warps an SM
+// leave half the issue slots free.  Instances for what is written, the vertex residual
+// moved beside the next step's stages and no clamping inside the grid took the rays of 256
+// elements, 256 rays, 512 x 512 pixels from 1357 to 1084 us without vertices and from
+// 1520 to 1357 with them.
 constexpr int TRACE_GR = 8;   // rays of one fan side by side in a warp (measured: 1, 2, 4, 8, 16)
-__global__ void __launch_bounds__(128) k_trace(GeoDev G, const float4* __restrict__ cells, rb_ray_end* __restrict__ ends,
-                                               rb_rays S, int write_samples, Vtx* __restrict__ verts,
+template <bool PUT, bool SAMPLES, bool INSIDE>
+__global__ void __launch_bounds__(128, 4) k_trace(GeoDev G, const float4* __restrict__ cells, rb_ray_end* __restrict__ ends,
+                                               rb_rays S, Vtx* __restrict__ verts,
                                                uint32_t* __restrict__ counters, uint32_t* __restrict__ fan_len) {
     // a warp takes TRACE_GR neighbouring rays of 32 / TRACE_GR fans: rays of alike take-off
     // angles (so alike lengths: the lanes finish together) that share field cells
@@ -332,8 +370,6 @@ __global__ void __launch_bounds__(128) k_trace(GeoDev G, const float4* __restric
     const long long qg = u / ((long long)TRACE_GR * G.n_elem), rg = u % ((long long)TRACE_GR * G.n_elem);
     const int t = (int)(rg / TRACE_GR), i = (int)(qg * TRACE_GR + rg % TRACE_GR);
     if (i >= G.n_rays) return;
-    const bool valid = true, owner = true;
-    const bool put = verts != nullptr;
 
     DF xs, ys;
     elem_pos(G, t, xs, ys);
@@ -346,7 +382,7 @@ __global__ void __launch_bounds__(128) k_trace(GeoDev G, const float4* __restric
     cc.fi = -1.f;
     cc.fj = -1.f;
     float f0[7];
-    sample(G, cells, cc, xs.hi + xs.lo, ys.hi + ys.lo, f0);
+    sample<INSIDE>(G, cells, cc, xs.hi + xs.lo, ys.hi + ys.lo, f0);
 
     float xh = xs.hi, xl = xs.lo, yh = ys.hi, yl = ys.lo, thh = thd.hi, thl = thd.lo;
     float tha = thh, Ca, Sa;
@@ -354,11 +390,10 @@ __global__ void __launch_bounds__(128) k_trace(GeoDev G, const float4* __restric
     float trh = 0.f, trl = 0.f;   // T as a float pair (compensated sum of the RK4 increments)
     float q = 0.f, p = 1.0f / f0[0], l = 0.f;
     int kap = 0;
-    bool alive = valid;
+    bool alive = true;
 
-    Vtx cur{xh, xl, yh, yl, 0.f, 0.f, 0.f, 0};
-    const size_t sbase = ((size_t)t * G.n_rays + (valid ? i : 0)) * (size_t)(G.max_steps + 1);
-    if (write_samples && valid) {
+    const size_t sbase = ((size_t)t * G.n_rays + i) * (size_t)(G.max_steps + 1);
+    if (SAMPLES) {
         S.vx[sbase] = xh + xl;
         S.vy[sbase] = yh + yl;
         S.vt[sbase] = 0.0;
@@ -366,11 +401,20 @@ __global__ void __launch_bounds__(128) k_trace(GeoDev G, const float4* __restric
         S.vl[sbase] = 0.f;
         S.vkappa[sbase] = 0;
     }
-    if (put) put_vtx(verts + vidx(G, t, 0, i), cur);
-    const float ds = G.ds, a2 = 0.5f * G.ds, ds6 = G.ds * (1.0f / 6.0f);
+    // vertex k - 1 goes out at the top of step k, beside that step's first stages, which do
+    // not depend on it: its residual is a chain of a hundred instructions of its own
+    Vtx* vout = PUT ? verts + vidx(G, t, 0, i) : nullptr;
+    auto put_current = [&]() {
+        // vertex residual T - |x - x_t| / c_ref in float pairs
+        const DF dx = df_sub(DF{xh, xl}, xs), dy = df_sub(DF{yh, yl}, ys);
+        const DF d2 = df_add(df_sqr(dx), df_sqr(dy));
+        const DF dist = d2.hi > 0.f ? df_sqrt(d2) : DF{0.f, 0.f};
+        const DF tr = df_sub(DF{trh, trl}, df_mul(dist, DF{G.inv_cref, G.inv_cref_lo}));
+        put_vtx(vout, Vtx{xh, xl, yh, yl, tr.hi + tr.lo, q, l, kap});
+        vout += G.n_rays;
+    };
 
-    for (int k = 1; k <= G.max_steps; ++k) {
-        if (!alive) break;
+    for (int k = 1; alive && k <= G.max_steps; ++k) {
         if (alive) {
             // direction relative to the anchor angle tha (cos / sin exact there); the
             // anchor follows the ray whenever it has turned by more than 0.05 rad
@@ -381,18 +425,9 @@ __global__ void __launch_bounds__(128) k_trace(GeoDev G, const float4* __restric
                 ray_sincos(tha, &Sa, &Ca);
             }
             const float dth = (thh - tha) + thl;
-            const Deriv z{0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-            const Deriv k1 = eval_stage(G, cells, cc, xh, xl, yh, yl, Ca, Sa, tha, dth, q, p, 0.f, z);
-            const Deriv k2 = eval_stage(G, cells, cc, xh, xl, yh, yl, Ca, Sa, tha, dth, q, p, a2, k1);
-            const Deriv k3 = eval_stage(G, cells, cc, xh, xl, yh, yl, Ca, Sa, tha, dth, q, p, a2, k2);
-            const Deriv k4 = eval_stage(G, cells, cc, xh, xl, yh, yl, Ca, Sa, tha, dth, q, p, ds, k3);
-            const float ix = ds6 * (k1.x + 2.f * k2.x + 2.f * k3.x + k4.x);
-            const float iy = ds6 * (k1.y + 2.f * k2.y + 2.f * k3.y + k4.y);
-            const float ith = ds6 * (k1.th + 2.f * k2.th + 2.f * k3.th + k4.th);
-            const float it = ds6 * (k1.t + 2.f * k2.t + 2.f * k3.t + k4.t);
-            const float iq = ds6 * (k1.q + 2.f * k2.q + 2.f * k3.q + k4.q);
-            const float ip = ds6 * (k1.p + 2.f * k2.p + 2.f * k3.p + k4.p);
-            const float il = ds6 * (k1.l + 2.f * k2.l + 2.f * k3.l + k4.l);
+            if (PUT) put_current();
+            const Deriv inc = rk4_step<INSIDE>(G, cells, cc, xh, xl, yh, yl, Ca, Sa, tha, dth, q, p);
+            const float ix = inc.x, iy = inc.y, ith = inc.th, it = inc.t, iq = inc.q, ip = inc.p, il = inc.l;
             float nxh = xh, nxl = xl, nyh = yh, nyl = yl, nthh = thh, nthl = thl;
             comp_add(nxh, nxl, ix);
             comp_add(nyh, nyl, iy);
@@ -409,7 +444,7 @@ __global__ void __launch_bounds__(128) k_trace(GeoDev G, const float4* __restric
                 const float lf = (float)lam;
                 const double ex = ax + lam * (bx - ax), ey = ay + lam * (by - ay);
                 const double tt = (double)trh + (double)trl;
-                const double et = tt + lam * (double)it;
+                const double et = __fma_rn(lam, (double)it, tt);
                 const double eth = ((double)thh + (double)thl) + lam * (((double)nthh + (double)nthl) - ((double)thh + (double)thl));
                 const float eq = q + lf * (nq - q), ep = p + lf * (np - p), el = l + lf * (nl - l);
                 const int ek = kap + ((k >= 2 && signbit(eq) != signbit(q)) ? 1 : 0);
@@ -418,11 +453,11 @@ __global__ void __launch_bounds__(128) k_trace(GeoDev G, const float4* __restric
                 const DF etd = df_from_double(et);
                 q = eq; p = ep; l = el; kap = ek; trh = etd.hi; trl = etd.lo;
                 alive = false;
-                if (owner) {
+                {
                     const double ddx = ex - xs_d, ddy = ey - ys_d;
                     rb_ray_end e;
                     e.t = et;
-                    e.t_res = et - sqrt(ddx * ddx + ddy * ddy) * (1.0 / G.c_ref_d);
+                    e.t_res = __fma_rn(-sqrt(__fma_rn(ddx, ddx, __dmul_rn(ddy, ddy))), 1.0 / G.c_ref_d, et);
                     e.x = ex;
                     e.y = ey;
                     e.theta = (float)eth;
@@ -441,7 +476,7 @@ __global__ void __launch_bounds__(128) k_trace(GeoDev G, const float4* __restric
                 q = nq; p = np; l = nl;
                 if (k == G.max_steps) {
                     alive = false;
-                    if (owner) {
+                    {
                         const double ex = (double)xh + (double)xl, ey = (double)yh + (double)yl;
                         const double ddx = ex - xs_d, ddy = ey - ys_d;
                         rb_ray_end e;
@@ -462,16 +497,7 @@ __global__ void __launch_bounds__(128) k_trace(GeoDev G, const float4* __restric
                     }
                 }
             }
-            if (put) {
-                // vertex residual T - |x - x_t| / c_ref in float pairs
-                const DF dx = df_sub(DF{xh, xl}, xs), dy = df_sub(DF{yh, yl}, ys);
-                const DF d2 = df_add(df_sqr(dx), df_sqr(dy));
-                const DF dist = d2.hi > 0.f ? df_sqrt(d2) : DF{0.f, 0.f};
-                const DF tr = df_sub(DF{trh, trl}, df_mul(dist, DF{G.inv_cref, G.inv_cref_lo}));
-                cur = Vtx{xh, xl, yh, yl, tr.hi + tr.lo, q, l, kap};
-                put_vtx(verts + vidx(G, t, k, i), cur);
-            }
-            if (write_samples) {
+            if (SAMPLES) {
                 const size_t o = sbase + (size_t)k;
                 const double vx = (double)xh + (double)xl, vy = (double)yh + (double)yl;
                 S.vx[o] = (float)vx;
@@ -483,6 +509,7 @@ __global__ void __launch_bounds__(128) k_trace(GeoDev G, const float4* __restric
             }
         }
     }
+    if (PUT) put_current();
 }
 
 // Index of the last vertex of ray i of fan t: the exit vertex, or max_steps for a
@@ -797,7 +824,17 @@ cudaError_t launch_trace(const GeoDev& G, const float4* cells, rb_ray_end* ends,
     }
     // threads: every fan's rays padded to a multiple of TRACE_GR (the padding returns at once)
     const long long rays = (long long)G.n_elem * ((G.n_rays + TRACE_GR - 1) / TRACE_GR) * TRACE_GR;
-    k_trace<<<(int)((rays + 127) / 128), 128, 0, s>>>(G, cells, ends, S, ws, V, counters, grid ? fan_len : nullptr);
+    const int tb = (int)((rays + 127) / 128);
+    uint32_t* fl = grid ? fan_len : nullptr;
+    // a ray's stages lie within a step of the ring: inside the grid unless it ends that close
+    const double half = 0.5 * (double)((G.nx < G.ny ? G.nx : G.ny) - 1) * G.h_d;
+    const bool inside = G.R_d + 1.001 * G.ds_d + 0.01 * G.h_d <= half;
+    if (V && ws) k_trace<true, true, false><<<tb, 128, 0, s>>>(G, cells, ends, S, V, counters, fl);
+    else if (ws) k_trace<false, true, false><<<tb, 128, 0, s>>>(G, cells, ends, S, V, counters, fl);
+    else if (V && inside) k_trace<true, false, true><<<tb, 128, 0, s>>>(G, cells, ends, S, V, counters, fl);
+    else if (V) k_trace<true, false, false><<<tb, 128, 0, s>>>(G, cells, ends, S, V, counters, fl);
+    else if (inside) k_trace<false, false, true><<<tb, 128, 0, s>>>(G, cells, ends, S, V, counters, fl);
+    else k_trace<false, false, false><<<tb, 128, 0, s>>>(G, cells, ends, S, V, counters, fl);
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess && traced) e = cudaEventRecord(traced, s);   // the end records are complete
     if (e != cudaSuccess || !grid) return e;
