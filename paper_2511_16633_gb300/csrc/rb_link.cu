@@ -67,6 +67,7 @@ __global__ void __launch_bounds__(256) k_link(GeoDev G, const float* __restrict_
     int* kk = (int*)(ll + n);                               // [n]
     int* ok = kk + n;                                       // [n]
     int* bi = ok + n;                                       // [N] winning interval per dr
+    float* crs = (float*)(bi + N);                          // [N] c at the receiver
     const int e = blockIdx.x;
     const double two_pi = 2.0 * RB_PI_D;
     const double phi_e = two_pi * (double)e / (double)N;
@@ -76,8 +77,9 @@ __global__ void __launch_bounds__(256) k_link(GeoDev G, const float* __restrict_
     ye *= G.R_d;
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
         const rb_ray_end E = ends[(size_t)e * n + i];
+        // in (-3 pi, pi]: the remainder by 2 pi is one exact addition where it is below -2 pi
         double a = atan2(E.y, E.x) - phi_e;
-        a = fmod(a, two_pi);
+        if (a <= -two_pi) a = __dadd_rn(a, two_pi);
         if (a < 0.0) a += two_pi;
         if (a >= two_pi) a -= two_pi;
         th[i] = a;
@@ -94,6 +96,7 @@ __global__ void __launch_bounds__(256) k_link(GeoDev G, const float* __restrict_
         xr *= G.R_d;
         yr *= G.R_d;
         cht[dr] = sqrt((xr - xe) * (xr - xe) + (yr - ye) * (yr - ye)) / G.c_ref_d;
+        if (F.n > 0) crs[dr] = bilinear_c(G, c, (float)xr, (float)yr);
         best[dr] = ~0ull;
         bi[dr] = 0x7fffffff;
     }
@@ -134,15 +137,11 @@ __global__ void __launch_bounds__(256) k_link(GeoDev G, const float* __restrict_
         const double bestT = bracket_T(cht[dr], th[bsel], th[bsel + 1], thr, tr[bsel], tr[bsel + 1], &bestLam);
         if (lrec) lrec[o] = LinkRec{bestT, bsel, (float)bestLam};
         if (F.n == 0) continue;
-        double xr, yr;
-        sincos(two_pi * (double)r / (double)N, &yr, &xr);
-        xr *= G.R_d;
-        yr *= G.R_d;
         const float lf = (float)bestLam;
         const float q = (1.f - lf) * qq[bsel] + lf * qq[bsel + 1];
         const float L = (1.f - lf) * ll[bsel] + lf * ll[bsel + 1];
         const int kap = bestLam <= 0.5 ? kk[bsel] : kk[bsel + 1];
-        const float crx = bilinear_c(G, c, (float)xr, (float)yr);
+        const float crx = crs[dr];
         const float J = fmaxf(fabsf(q), G.j_floor);
         for (int w = 0; w < F.n; ++w) {
             const FreqC& fc = F.f[w];
@@ -382,7 +381,7 @@ __global__ void k_sel_write(int n_total, const uint64_t* __restrict__ keys, cons
 cudaError_t launch_link(const GeoDev& G, const float* c, const rb_ray_end* ends, const FreqSet& F, float2* p_out,
                         uint8_t* linked, cudaStream_t s, LinkRec* lrec) {
     if (G.n_rays > LINK_MAX_RAYS) return cudaErrorInvalidValue;
-    const size_t sm = (size_t)G.n_rays * (8 + 8 + 4 + 4 + 4 + 4) + (size_t)G.n_elem * (8 + 8 + 4);
+    const size_t sm = (size_t)G.n_rays * (8 + 8 + 4 + 4 + 4 + 4) + (size_t)G.n_elem * (8 + 8 + 4 + 4);
     if (sm > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(k_link, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
         if (e != cudaSuccess) return e;
