@@ -281,8 +281,7 @@ rb_status gradient_stages(const GeoDev& G, const FreqSet& F, const Ws& W, float*
     const Marks mark2{mark.ev, s2};   // stage events of the side branch
     RB_CU(cudaMemsetAsync(cnt, 0, CNT_N * 4 + DBL_N * 8, s));
     RB_CU(mark(RB_STAGE_FIELDS, 0));
-    RB_CU(launch_elem_positions(G, exy, s));
-    RB_CU(launch_fields(G, c, alpha0, cells, s));
+    RB_CU(launch_fields(G, c, alpha0, cells, exy, s));
     // side branch 1: the first-arrival keys reset (all ones) beside the tracer; forked
     // after the fields, which it would otherwise slow (0.098 against 0.031 ms on a
     // 256-element ring at 512^2 pixels), by a fill of one CTA per SM
@@ -413,8 +412,7 @@ rb_status rb_trace_rays(const rb_geometry* geom, const float* c, const float* al
     uint32_t* cnt = W.at<uint32_t>(W.L.counters);
     const GeoDev G = make_geo(geom, exy);
     RB_CU(cudaMemsetAsync(cnt, 0, CNT_N * 4, s));
-    RB_CU(launch_elem_positions(G, exy, s));
-    RB_CU(launch_fields(G, c, alpha0, W.at<float4>(W.L.cells), s));
+    RB_CU(launch_fields(G, c, alpha0, W.at<float4>(W.L.cells), exy, s));
     RB_CU(launch_trace(G, W.at<float4>(W.L.cells), out->ends, out, nullptr, nullptr, nullptr, nullptr, cnt, s));
     return RB_OK;
 }
@@ -436,8 +434,7 @@ rb_status rb_green_grid(const rb_geometry* geom, const float* c, const float* al
     uint32_t* cnt = W.at<uint32_t>(W.L.counters);
     const GeoDev G = make_geo(geom, exy);
     RB_CU(cudaMemsetAsync(cnt, 0, CNT_N * 4, s));
-    RB_CU(launch_elem_positions(G, exy, s));
-    RB_CU(launch_fields(G, c, alpha0, W.at<float4>(W.L.cells), s));
+    RB_CU(launch_fields(G, c, alpha0, W.at<float4>(W.L.cells), exy, s));
     RB_CU(launch_trace(G, W.at<float4>(W.L.cells), W.at<rb_ray_end>(W.L.ends), nullptr, W.at<void>(W.L.gkeys), tables,
                        W.at<void>(W.L.verts), nullptr, cnt, s, nullptr, nullptr, nullptr, nullptr, 0,
                        W.at<uint32_t>(W.L.fanlen)));
@@ -475,8 +472,7 @@ rb_status rb_data_weights(const rb_geometry* geom, const float* c, const float* 
     uint8_t* linked = W.at<uint8_t>(W.L.linked);
     float2* R = (float2*)resid_out;
     RB_CU(cudaMemsetAsync(cnt, 0, CNT_N * 4, s));
-    RB_CU(launch_elem_positions(G, exy, s));
-    RB_CU(launch_fields(G, c, alpha0, W.at<float4>(W.L.cells), s));
+    RB_CU(launch_fields(G, c, alpha0, W.at<float4>(W.L.cells), exy, s));
     RB_CU(launch_trace(G, W.at<float4>(W.L.cells), ends, nullptr, nullptr, nullptr, nullptr, nullptr, cnt, s));
     RB_CU(launch_link(G, c, ends, F, R, linked, s));
     RB_CU(launch_residual_keys(G, n_freq, (const float2*)p_obs, R, linked, W.at<uint64_t>(W.L.keys), cnt,
@@ -578,7 +574,7 @@ rb_status rb_hf_update(const rb_geometry* geom, float* c_inout, const float* alp
     float2* fwd = W.at<float2>(W.L.fwd);
     const int nch = rb_fwd_chunks_for(G.n_elem, G.npix);
     RB_CU(mark(RB_STAGE_DIRECTION, 0));
-    RB_CU(launch_update(G, c_inout, gsum, hsum, pdir, dc_out, part, dbl, cnt, diag_out, params->eps_rel,
+    RB_CU(launch_update(G, c_inout, gsum, hsum, pdir, dc_out, part, n_freq, dbl, cnt, diag_out, params->eps_rel,
                         params->step_mode, 0, s));
     RB_CU(mark(RB_STAGE_DIRECTION, 1));
     RB_CU(mark(RB_STAGE_FORWARD, 0));
@@ -606,12 +602,11 @@ rb_status rb_hf_update(const rb_geometry* geom, float* c_inout, const float* alp
                                             part + (size_t)w * 256, s));
             }
         }
-        RB_CU(launch_sum_partials(part, n_freq * 256, dbl, DBL_DEN, 1.0, 0, s));
     }
     RB_CU(mark(RB_STAGE_FORWARD, 1));
     RB_CU(mark(RB_STAGE_APPLY, 0));
-    RB_CU(launch_update(G, c_inout, gsum, hsum, pdir, dc_out, part + (size_t)RB_MAX_FREQ * 256, dbl, cnt, diag_out,
-                        params->eps_rel, params->step_mode, 1, s, limit_word));
+    RB_CU(launch_update(G, c_inout, gsum, hsum, pdir, dc_out, part, n_freq, dbl, cnt, diag_out, params->eps_rel,
+                        params->step_mode, 1, s, limit_word));
     RB_CU(mark(RB_STAGE_APPLY, 1));
     return RB_OK;
 }
@@ -682,8 +677,8 @@ rb_status rb_cg_update(const rb_geometry* geom, float* c_inout, const float* alp
     if (cg_hist_out) RB_CU(launch_cg_history(dbl, cg_iters, cg_hist_out, s));
     RB_CU(mark(RB_STAGE_FORWARD, 1));
     RB_CU(mark(RB_STAGE_APPLY, 0));
-    RB_CU(launch_update(G, c_inout, gsum, hsum, x, dc_out, vpart, dbl, cnt, diag_out, params->eps_rel, RB_STEP_DIAG,
-                        1, s, limit_word));
+    RB_CU(launch_update(G, c_inout, gsum, hsum, x, dc_out, part, n_freq, dbl, cnt, diag_out, params->eps_rel,
+                        RB_STEP_DIAG, 1, s, limit_word));
     RB_CU(mark(RB_STAGE_APPLY, 1));
     return RB_OK;
 }
@@ -701,8 +696,7 @@ rb_status rb_tof_times(const rb_geometry* geom, const float* c, const float* alp
     const GeoDev G = make_geo(geom, exy);
     rb_ray_end* ends = W.at<rb_ray_end>(W.L.ends);
     RB_CU(cudaMemsetAsync(cnt, 0, CNT_N * 4, s));
-    RB_CU(launch_elem_positions(G, exy, s));
-    RB_CU(launch_fields(G, c, alpha0, W.at<float4>(W.L.cells), s));
+    RB_CU(launch_fields(G, c, alpha0, W.at<float4>(W.L.cells), exy, s));
     RB_CU(launch_trace(G, W.at<float4>(W.L.cells), ends, nullptr, nullptr, nullptr, nullptr, nullptr, cnt, s));
     RB_CU(launch_tof_link(G, c, ends, W.at<void>(W.L.tof), linked_out, s));
     RB_CU(launch_tof_times_out(G, W.at<void>(W.L.tof), t_out, s));
@@ -728,10 +722,9 @@ rb_status rb_tof_invert(const rb_geometry* geom, float* c_inout, const float* al
     Vtx* verts = W.at<Vtx>(W.L.verts);
     double* part = W.at<double>(W.L.part);
     RB_CU(cudaMemsetAsync(cnt, 0, CNT_N * 4, s));
-    RB_CU(launch_elem_positions(G, exy, s));
     for (int k = 0; k <= n_iter; ++k) {
         const bool last = k == n_iter;
-        RB_CU(launch_fields(G, c_inout, alpha0, cells, s));
+        RB_CU(launch_fields(G, c_inout, alpha0, cells, k == 0 ? exy : nullptr, s));
         RB_CU(launch_trace(G, cells, ends, nullptr, nullptr, nullptr, last ? nullptr : (void*)verts, nullptr, cnt, s));
         RB_CU(launch_tof_link(G, c_inout, ends, tw, nullptr, s));
         if (resid_out) RB_CU(launch_tof_resid(G, tw, t_obs, obs_linked, part, resid_out + k, s));

@@ -323,15 +323,30 @@ __device__ uint64_t sel_resolve(const uint64_t* src, int n, uint64_t prefix, lon
             if (key != 0 && (key & mask) == pre) atomicAdd(&hist[(key >> sh) & dm], 1u);
         }
         __syncthreads();
-        if (threadIdx.x == 0) {
-            long long r = s_rem;
-            int d = (int)dm;
-            for (; d > 0; --d) {
-                if ((long long)hist[d] >= r) break;
-                r -= hist[d];
+        if (threadIdx.x < 32) {
+            // the digit that holds the s_rem-th largest: lane l's bins 8 l .. 8 l + 7, suffix sums
+            // over the lanes (by one thread this search was most of the kernel's 27 to 39 us)
+            const long long r = s_rem;
+            uint32_t h[8], own = 0;
+#pragma unroll
+            for (int q = 0; q < 8; ++q) own += h[q] = hist[8 * threadIdx.x + q];
+            uint32_t incl = own;
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t u = __shfl_down_sync(0xffffffffu, incl, o);
+                if (threadIdx.x + o < 32) incl += u;
             }
-            s_rem = r;
-            s_prefix = pre | ((uint64_t)d << sh);
+            const uint32_t above = incl - own;
+            if ((long long)above < r && (r <= (long long)incl || threadIdx.x == 0)) {
+                long long left = r - above;
+                int d = 8 * (int)threadIdx.x;
+                for (int q = 7; q >= 0; --q) {
+                    d = 8 * (int)threadIdx.x + q;
+                    if ((long long)h[q] >= left || d == 0) break;
+                    left -= h[q];
+                }
+                s_rem = left;
+                s_prefix = pre | ((uint64_t)d << sh);
+            }
         }
         mask |= dm << sh;
         __syncthreads();

@@ -46,21 +46,33 @@ __global__ void __launch_bounds__(RT) k_hsum_part(GeoDev G, const float* __restr
     block_sum_store(cnt, part + RB + blockIdx.x);
 }
 
-__global__ void __launch_bounds__(RT) k_eps(const double* __restrict__ part, double eps_rel, double* __restrict__ dbl) {
-    __shared__ double s[RT], t[RT];
-    s[threadIdx.x] = part[threadIdx.x];
-    t[threadIdx.x] = part[RB + threadIdx.x];
+// Sum of n partials over a block's RT threads in a fixed tree, handed to every thread.  The
+// scalars of an update are needed by whole grids: each block sums the partials itself (the
+// same tree, so the same bits, in every block) instead of waiting for a one-block kernel, 3 to
+// 4 us each of which nearly all was launch and tail.
+__device__ __forceinline__ double block_sum_all(const double* __restrict__ part, int n) {
+    __shared__ double s[RT];
+    double acc = 0.0;
+    for (int i = threadIdx.x; i < n; i += RT) acc += part[i];
+    __syncthreads();   // s may still be read from an earlier call
+    s[threadIdx.x] = acc;
     __syncthreads();
     for (int k = RT / 2; k > 0; k >>= 1) {
-        if (threadIdx.x < k) {
-            s[threadIdx.x] += s[threadIdx.x + k];
-            t[threadIdx.x] += t[threadIdx.x + k];
-        }
+        if (threadIdx.x < k) s[threadIdx.x] += s[threadIdx.x + k];
         __syncthreads();
     }
-    if (threadIdx.x == 0) {
-        dbl[DBL_HMEAN] = t[0] > 0.0 ? s[0] / t[0] : 0.0;
-        dbl[DBL_EPS] = eps_rel * dbl[DBL_HMEAN];
+    return s[0];
+}
+
+// mean of H over the support and eps from k_hsum_part's partials; block 0 records them
+__device__ __forceinline__ void hmean_eps(const double* __restrict__ hpart, double eps_rel, double* __restrict__ dbl,
+                                          double& hmean, double& eps) {
+    const double hs = block_sum_all(hpart, RB), cnt = block_sum_all(hpart + RB, RB);
+    hmean = cnt > 0.0 ? hs / cnt : 0.0;
+    eps = eps_rel * hmean;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        dbl[DBL_HMEAN] = hmean;
+        dbl[DBL_EPS] = eps;
     }
 }
 
@@ -81,9 +93,12 @@ __global__ void __launch_bounds__(RT) k_sum_part(const double* __restrict__ part
 
 // phase 1: direction p and partials of -<g, p>
 __global__ void __launch_bounds__(RT) k_direction(GeoDev G, const float* __restrict__ gsum, const float* __restrict__ hsum,
-                                                  const double* __restrict__ dbl, float* __restrict__ pdir,
+                                                  const double* __restrict__ hpart, double eps_rel,
+                                                  double* __restrict__ dbl, float* __restrict__ pdir,
                                                   double* __restrict__ part) {
-    const float eps = (float)dbl[DBL_EPS];
+    double hm_d, eps_d;
+    hmean_eps(hpart, eps_rel, dbl, hm_d, eps_d);
+    const float eps = (float)eps_d;
     double acc = 0.0;
     for (int p = blockIdx.x * RT + threadIdx.x; p < G.npix; p += RB * RT) {
         float v = 0.f;
@@ -97,14 +112,16 @@ __global__ void __launch_bounds__(RT) k_direction(GeoDev G, const float* __restr
     block_sum_store(acc, part + blockIdx.x);
 }
 
-// phase 2: alpha, dc, c update and partials of ||dc||^2
+// phase 2: alpha from the partials of -<g, p> (num_part) and of the n_den blocks of
+// sum W |B p|^2 (den_part), dc, c update and partials of ||dc||^2
 __global__ void __launch_bounds__(RT) k_apply(GeoDev G, float* __restrict__ c, const float* __restrict__ pdir,
-                                              double* __restrict__ dbl, int step_mode, float* __restrict__ dc_out,
-                                              double* __restrict__ part) {
+                                              const double* __restrict__ num_part, const double* __restrict__ den_part,
+                                              int n_den, double* __restrict__ dbl, int step_mode,
+                                              float* __restrict__ dc_out, double* __restrict__ part) {
     double alpha = 1.0;
     if (step_mode == RB_STEP_EXACT) {
-        const double den = dbl[DBL_DEN];
-        alpha = den > 0.0 ? dbl[DBL_NUM] / den : 0.0;
+        const double num = block_sum_all(num_part, RB), den = block_sum_all(den_part, n_den);
+        alpha = den > 0.0 ? num / den : 0.0;
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) dbl[DBL_ALPHA] = alpha;
     const float af = (float)alpha;
@@ -135,9 +152,12 @@ __device__ __forceinline__ float cg_minv(const float* __restrict__ hsum, int p, 
 }
 
 __global__ void __launch_bounds__(RT) k_cg_init(GeoDev G, const float* __restrict__ gsum, const float* __restrict__ hsum,
-                                                const double* __restrict__ dbl, int precond, float* __restrict__ x,
+                                                const double* __restrict__ hpart, double eps_rel,
+                                                double* __restrict__ dbl, int precond, float* __restrict__ x,
                                                 float* __restrict__ r, float* __restrict__ pv, double* __restrict__ part) {
-    const float eps = (float)dbl[DBL_EPS], hm = (float)dbl[DBL_HMEAN];
+    double hm_d, eps_d;
+    hmean_eps(hpart, eps_rel, dbl, hm_d, eps_d);
+    const float eps = (float)eps_d, hm = (float)hm_d;
     double acc = 0.0;
     for (int p = blockIdx.x * RT + threadIdx.x; p < G.npix; p += RB * RT) {
         float rv = 0.f, zv = 0.f;
@@ -183,15 +203,18 @@ __global__ void __launch_bounds__(RT) k_cg_p(GeoDev G, const float* __restrict__
         if (in_support(G, p)) pv[p] = fmaf(beta, pv[p], cg_minv(hsum, p, precond, eps, hm) * r[p]);
 }
 
-// The diagnostics record (when asked for), and the lost-ray count into the caller
-// stream's host-mapped limit word when rays were lost (read by the next update call).
-__global__ void k_finish(const double* __restrict__ dbl, const uint32_t* __restrict__ cnt, rb_diag* __restrict__ diag,
-                         uint32_t* __restrict__ limit_word) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
+// The diagnostics record (when asked for; ||dc||^2 from k_apply's partials), and the lost-ray
+// count into the caller stream's host-mapped limit word when rays were lost (read by the next
+// update call).
+__global__ void __launch_bounds__(RT) k_finish(const double* __restrict__ dbl, const double* __restrict__ norm_part,
+                                               const uint32_t* __restrict__ cnt, rb_diag* __restrict__ diag,
+                                               uint32_t* __restrict__ limit_word) {
+    const double norm2 = block_sum_all(norm_part, RB);
+    if (threadIdx.x != 0) return;
     if (limit_word && cnt[CNT_LOST] > 0) *(volatile uint32_t*)limit_word = cnt[CNT_LOST];
     if (!diag) return;
     rb_diag d;
-    d.dc_norm = sqrt(dbl[DBL_NORM2]);
+    d.dc_norm = sqrt(norm2);
     d.alpha = dbl[DBL_ALPHA];
     d.eps = dbl[DBL_EPS];
     d.lost_rays = cnt[CNT_LOST];
@@ -205,22 +228,23 @@ __global__ void k_finish(const double* __restrict__ dbl, const uint32_t* __restr
 
 }  // namespace
 
-// Launch sequence pieces used by rb_hf_update (rb_api.cu).
+// Launch sequence pieces used by rb_hf_update (rb_api.cu).  part: (RB_MAX_FREQ + 2) x RB
+// partials; rows 0 .. n_freq - 1 hold those of sum W |B p|^2 between the two phases, rows 0
+// and 1 H's before that, row RB_MAX_FREQ those of -<g, p> and row RB_MAX_FREQ + 1 ||dc||^2's.
 cudaError_t launch_update(const GeoDev& G, float* c, const float* gsum, const float* hsum, float* pdir, float* dc_out,
-                          double* part, double* dbl, uint32_t* counters, rb_diag* diag, double eps_rel, int step_mode,
-                          int phase, cudaStream_t s, uint32_t* limit_word) {
+                          double* part, int n_freq, double* dbl, uint32_t* counters, rb_diag* diag, double eps_rel,
+                          int step_mode, int phase, cudaStream_t s, uint32_t* limit_word) {
+    double* num = part + (size_t)RB_MAX_FREQ * RB;
+    double* norm = num + RB;
     switch (phase) {
         case 0: {  // eps, direction, numerator
             k_hsum_part<<<RB, RT, 0, s>>>(G, hsum, part);
-            k_eps<<<1, RT, 0, s>>>(part, eps_rel, dbl);
-            k_direction<<<RB, RT, 0, s>>>(G, gsum, hsum, dbl, pdir, part);
-            k_sum_part<<<1, RT, 0, s>>>(part, RB, dbl, DBL_NUM, 1.0, 0);
+            k_direction<<<RB, RT, 0, s>>>(G, gsum, hsum, part, eps_rel, dbl, pdir, num);
             break;
         }
         case 1: {  // apply the step and finish
-            k_apply<<<RB, RT, 0, s>>>(G, c, pdir, dbl, step_mode, dc_out, part);
-            k_sum_part<<<1, RT, 0, s>>>(part, RB, dbl, DBL_NORM2, 1.0, 0);
-            if (diag || limit_word) k_finish<<<1, 32, 0, s>>>(dbl, counters, diag, limit_word);
+            k_apply<<<RB, RT, 0, s>>>(G, c, pdir, num, part, n_freq * RB, dbl, step_mode, dc_out, norm);
+            if (diag || limit_word) k_finish<<<1, RT, 0, s>>>(dbl, norm, counters, diag, limit_word);
             break;
         }
         default:
@@ -232,9 +256,9 @@ cudaError_t launch_update(const GeoDev& G, float* c, const float* gsum, const fl
 cudaError_t launch_cg_init(const GeoDev& G, const float* gsum, const float* hsum, int precond, float* x, float* r,
                            float* p, double* part, double* dbl, double eps_rel, cudaStream_t s) {
     k_hsum_part<<<RB, RT, 0, s>>>(G, hsum, part);
-    k_eps<<<1, RT, 0, s>>>(part, eps_rel, dbl);
-    k_cg_init<<<RB, RT, 0, s>>>(G, gsum, hsum, dbl, precond, x, r, p, part);
-    k_sum_part<<<1, RT, 0, s>>>(part, RB, dbl, DBL_CG_RHO, 1.0, 0);
+    double* rpart = part + 2 * RB;   // H's partials are read by every block of k_cg_init
+    k_cg_init<<<RB, RT, 0, s>>>(G, gsum, hsum, part, eps_rel, dbl, precond, x, r, p, rpart);
+    k_sum_part<<<1, RT, 0, s>>>(rpart, RB, dbl, DBL_CG_RHO, 1.0, 0);
     return cudaGetLastError();
 }
 
