@@ -436,9 +436,8 @@ rb_status rb_green_grid(const rb_geometry* geom, const float* c, const float* al
     RB_CU(cudaMemsetAsync(cnt, 0, CNT_N * 4, s));
     RB_CU(launch_fields(G, c, alpha0, W.at<float4>(W.L.cells), exy, s));
     RB_CU(launch_trace(G, W.at<float4>(W.L.cells), W.at<rb_ray_end>(W.L.ends), nullptr, W.at<void>(W.L.gkeys), tables,
-                       W.at<void>(W.L.verts), nullptr, cnt, s, nullptr, nullptr, nullptr, nullptr, 0,
-                       W.at<uint32_t>(W.L.fanlen)));
-    if (g_out) RB_CU(launch_green_out(G, tables, c, F, (float2*)g_out, s));
+                       W.at<void>(W.L.verts), c, cnt, s, nullptr, nullptr, g_out ? &F : nullptr, nullptr, 0,
+                       W.at<uint32_t>(W.L.fanlen), (float2*)g_out));
     return RB_OK;
 }
 

@@ -351,32 +351,25 @@ __global__ void __launch_bounds__(256) k_forward_reduce(GeoDev G, FreqC F, const
     }
 }
 
-// Green's functions written out, g[w][t][pixel] (tests and users who want G itself).
-__global__ void k_green_out(GeoDev G, const rb_cell* __restrict__ tables, const float* __restrict__ c, FreqSet F,
-                            float2* __restrict__ g) {
-    const long long total = (long long)G.n_elem * G.npix;
-    for (long long j = blockIdx.x * (long long)blockDim.x + threadIdx.x; j < total; j += (long long)gridDim.x * blockDim.x) {
-        const int t = (int)(j / G.npix), pix = (int)(j % G.npix);
-        const rb_cell rec = tables[j];
-        const int ix = pix % G.nx, iy = pix / G.nx;
+// Green's functions of one frequency from the tables, g[t][pixel], for the plain forward.
+// Bound by the 24 bytes an entry it reads and writes; a CTA stays on 256 pixels and goes
+// through the elements with the grid's second dimension, so that neither the entry's index
+// nor the pixel's row takes a division per entry.
+__global__ void __launch_bounds__(256) k_green_out(GeoDev G, const rb_cell* __restrict__ tables,
+                                                   const float* __restrict__ c, FreqC F, float2* __restrict__ g) {
+    const int pix = blockIdx.x * blockDim.x + threadIdx.x;
+    if (pix >= G.npix) return;
+    const int iy = pix / G.nx, ix = pix - iy * G.nx;
+    const float cv = __ldg(c + pix);
+    for (int t = blockIdx.y; t < G.n_elem; t += gridDim.y) {
+        const size_t j = (size_t)t * G.npix + pix;
         DF ex, ey;
         elem_pos(G, t, ex, ey);
-        const DF dist = pixel_elem_dist(G, ix, iy, ex, ey);
-        const float cv = __ldg(c + pix);
-        for (int w = 0; w < F.n; ++w) g[(size_t)w * total + j] = green_eval(rec, cv, dist, F.f[w], G.j_floor);
+        g[j] = green_eval(tables[j], cv, pixel_elem_dist(G, ix, iy, ex, ey), F, G.j_floor);
     }
 }
 
 }  // namespace
-
-cudaError_t launch_green_out(const GeoDev& G, const rb_cell* tables, const float* c, const FreqSet& F, float2* g_out,
-                             cudaStream_t s) {
-    const long long total = (long long)G.n_elem * G.npix;
-    long long blocks = (total + 255) / 256;
-    if (blocks > 4096) blocks = 4096;
-    k_green_out<<<(int)blocks, 256, 0, s>>>(G, tables, c, F, g_out);
-    return cudaGetLastError();
-}
 
 size_t simt_sym_bytes(int n_elem) {
     const size_t np = (size_t)((n_elem + EB - 1) / EB) * EB;
@@ -420,10 +413,11 @@ cudaError_t launch_forward_simt(const GeoDev& G, const rb_cell* tables, const fl
         k_forward_simt<false><<<grid, FTHR, 0, s>>>(G, nullptr, tables, c, F, m, partial, n_chunks);
         return cudaGetLastError();
     }
-    FreqSet F1;
-    F1.n = 1;
-    F1.f[0] = F;
-    cudaError_t e = launch_green_out(G, tables, c, F1, g_buf, s);
+    const int bx = (G.npix + 255) / 256;
+    int by = (4864 + bx - 1) / bx;   // 32 CTAs an SM: four waves of eight
+    if (by > G.n_elem) by = G.n_elem;
+    k_green_out<<<dim3(bx, by), 256, 0, s>>>(G, tables, c, F, g_buf);
+    cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     k_forward_simt<true><<<grid, FTHR, 0, s>>>(G, g_buf, tables, c, F, m, partial, n_chunks);
     return cudaGetLastError();

@@ -684,10 +684,14 @@ __device__ __forceinline__ bool resolve_entry(const GeoDev& G, const Vtx* __rest
 // Thread = pixel (its coordinates and support test computed once), looping over the
 // elements t = blockIdx.y, blockIdx.y + gridDim.y, ...; consecutive threads take
 // consecutive pixels, so every key load and record store is coalesced.
+// GREEN: the Green's functions of the set go out with the records, g[w][t][pixel].
+template <bool GREEN>
 __global__ void __launch_bounds__(256) k_resolve(GeoDev G, const Vtx* __restrict__ verts,
                                                  const rb_ray_end* __restrict__ ends,
                                                  const unsigned long long* __restrict__ keys, rb_cell* __restrict__ tables,
-                                                 uint32_t* __restrict__ counters, uint32_t kq_magic) {
+                                                 uint32_t* __restrict__ counters, uint32_t kq_magic,
+                                                 const float* __restrict__ c, const __grid_constant__ FreqSet F,
+                                                 float2* __restrict__ g) {
     uint32_t holes = 0;   // support pixels that no triangle of the fan covered
     for (int pix = blockIdx.x * blockDim.x + threadIdx.x; pix < G.npix; pix += gridDim.x * blockDim.x) {
         const int iy = pix / G.nx, ix = pix - iy * G.nx;
@@ -695,10 +699,14 @@ __global__ void __launch_bounds__(256) k_resolve(GeoDev G, const Vtx* __restrict
         const DF Y = df_pixel_coord(iy, G.cyg, G.h_hi, G.h_lo);
         const long long jx = 2LL * ix - (G.nx - 1), jy = 2LL * iy - (G.ny - 1);
         const bool in_support = jx * jx + jy * jy <= G.r2max;
+        const float c_px = GREEN ? __ldg(c + pix) : 0.f;
+        unsigned long long next = (int)blockIdx.y < G.n_elem ? keys[(size_t)blockIdx.y * G.npix + pix] : ~0ull;
         for (int t = blockIdx.y; t < G.n_elem; t += gridDim.y) {
             const size_t u = (size_t)t * G.npix + pix;
+            const unsigned long long key = next;   // the next element's is on its way meanwhile
+            if (t + (int)gridDim.y < G.n_elem) next = keys[u + (size_t)gridDim.y * G.npix];
             rb_cell rec;
-            if (!resolve_entry(G, verts, ends, keys[u], t, X, Y, kq_magic, rec)) {
+            if (!resolve_entry(G, verts, ends, key, t, X, Y, kq_magic, rec)) {
                 rec.tag = RB_HOLE;
                 rec.tkey = RB_HOLE;
                 rec.q = __uint_as_float(RB_HOLE);
@@ -706,6 +714,13 @@ __global__ void __launch_bounds__(256) k_resolve(GeoDev G, const Vtx* __restrict
                 if (in_support) ++holes;
             }
             tables[u] = rec;
+            if (GREEN) {
+                DF ex, ey;
+                elem_pos(G, t, ex, ey);
+                const DF dist = pixel_elem_dist(G, ix, iy, ex, ey);
+                for (int w = 0; w < F.n; ++w)
+                    g[((size_t)w * G.n_elem + t) * G.npix + pix] = green_eval(rec, c_px, dist, F.f[w], G.j_floor);
+            }
         }
     }
     for (int o = 16; o > 0; o >>= 1) holes += __shfl_down_sync(0xffffffffu, holes, o);
@@ -799,7 +814,7 @@ cudaError_t launch_keys_reset(const GeoDev& G, void* keys, cudaStream_t s) {
 cudaError_t launch_trace(const GeoDev& G, const float4* cells, rb_ray_end* ends, const rb_rays* samples,
                          void* keys, rb_cell* tables, void* verts, const float* c, uint32_t* counters,
                          cudaStream_t s, cudaEvent_t traced, cudaEvent_t keys_ready, const FreqSet* F, void* images,
-                         int raster_mode, uint32_t* fan_len) {
+                         int raster_mode, uint32_t* fan_len, float2* green) {
     rb_rays S{};
     int ws = 0;
     if (samples && samples->vx) {
@@ -813,6 +828,7 @@ cudaError_t launch_trace(const GeoDev& G, const float4* cells, rb_ray_end* ends,
     const bool fused = images != nullptr;
     if (fused && (!F || F->n < 1 || !c || (G.n_elem % 16) != 0)) return cudaErrorInvalidValue;
     if (grid && (!V || (!tables && !fused))) return cudaErrorInvalidValue;
+    if (green && (!tables || !F || F->n < 1 || !c)) return cudaErrorInvalidValue;
     unsigned long long* K = (unsigned long long*)keys;
     if (grid && !keys_ready) {
         cudaError_t e = cudaMemsetAsync(K, 0xff, (size_t)G.n_elem * G.npix * sizeof(unsigned long long), s);
@@ -872,7 +888,10 @@ cudaError_t launch_trace(const GeoDev& G, const float4* cells, rb_ray_end* ends,
     int bx = (G.npix + 255) / 256;
     int by = 1;
     while (by < 16 && by * 2 <= G.n_elem && (long long)bx * by < (long long)nsm * 16) by *= 2;
-    k_resolve<<<dim3(bx, by), 256, 0, s>>>(G, V, ends, K, tables, counters, kq_magic);
+    if (green)
+        k_resolve<true><<<dim3(bx, by), 256, 0, s>>>(G, V, ends, K, tables, counters, kq_magic, c, *F, green);
+    else
+        k_resolve<false><<<dim3(bx, by), 256, 0, s>>>(G, V, ends, K, tables, counters, kq_magic, c, FreqSet{}, nullptr);
     return cudaGetLastError();
 }
 

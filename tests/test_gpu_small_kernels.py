@@ -10,6 +10,8 @@ pytestmark = pytest.mark.gpu
 
 import rbgen  # noqa: E402
 from oracle import geometry as ogeom  # noqa: E402
+from oracle import green as ogreen  # noqa: E402
+from oracle import grid as ogrid  # noqa: E402
 from oracle import rays as orays  # noqa: E402
 from oracle.rays import VTH, VX, VY  # noqa: E402
 from paper_2511_16633_gb300 import rb  # noqa: E402
@@ -80,3 +82,26 @@ def test_outlier_selection_digits(dev, kind, frac):
     want = kept.copy()
     want[order[:k]] = False
     assert np.array_equal(W == 1, want)
+
+
+@pytest.mark.parametrize("nx,ny,n_elem,n_freq", [(65, 67, 9, 1), (64, 64, 17, 3), (71, 66, 33, 2)])
+def test_green_with_tables(dev, nx, ny, n_elem, n_freq):
+    """Green's functions written with the tables: the tables of the call without them, and the
+    oracle's values within 1e-4 (relative L2, the plain path's bound)."""
+    cfg = rbgen.tiny(nx=nx, ny=ny, n_elem=n_elem)
+    inp = rbgen.make_inputs(rbgen.tiny(nx=nx, ny=ny, seed=cfg.seed))
+    geom = rb.geometry_from_config(cfg)
+    c, a0 = _t(inp.c_true, dev), _t(inp.alpha0, dev)
+    ws = rb.workspace(geom, 1, rb.RB_PREC_FP32, dev)
+    freqs = [cfg.freqs_hz[0] * (1 + 0.3 * k) for k in range(n_freq)]
+    tabs = [torch.empty((n_elem, nx * ny, 4), dtype=torch.int32, device=dev) for _ in range(2)]
+    g_out = torch.empty((n_freq, n_elem, nx * ny), dtype=torch.complex64, device=dev)
+    rb.rb_green_grid(geom, c, a0, tabs[0], ws)
+    rb.rb_green_grid(geom, c, a0, tabs[1], ws, freqs, g_out)
+    assert torch.equal(tabs[0], tabs[1])
+    g = ogeom.from_config(cfg)
+    ot = ogrid.grid(g, inp.c_true, inp.alpha0)
+    for j, f in enumerate(freqs):
+        want = np.ravel(ogreen.green(g, ot, inp.c_true, f))
+        got = np.ravel(g_out[j].cpu().numpy())
+        assert np.linalg.norm(got - want) <= 1e-4 * np.linalg.norm(want)
