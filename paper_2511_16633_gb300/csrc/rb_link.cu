@@ -53,6 +53,9 @@ __device__ __forceinline__ unsigned long long d2key(double v) {
 // order-preserving 64-bit traveltime key (shared-memory atomic min), ties to the
 // smallest interval index in a second pass, which reproduces a sequential scan
 // over i that keeps the first strictly smaller T.
+// Bound by double arithmetic (two lanes a cycle and SM): the end angles' atan2, then the
+// receivers looked at.  Their angles are formed once per CTA: a division for each of the
+// three or four receivers that an interval looks at, in both passes, was most of it.
 __global__ void __launch_bounds__(256) k_link(GeoDev G, const float* __restrict__ c, const rb_ray_end* __restrict__ ends,
                                               FreqSet F, float2* __restrict__ p_out, uint8_t* __restrict__ linked,
                                               LinkRec* __restrict__ lrec) {
@@ -61,7 +64,8 @@ __global__ void __launch_bounds__(256) k_link(GeoDev G, const float* __restrict_
     double* th = (double*)smem;                             // [n]
     double* tr = th + n;                                    // [n]
     double* cht = tr + n;                                   // [N] chord / c_ref per receiver offset dr
-    unsigned long long* best = (unsigned long long*)(cht + N);   // [N] first-arrival key per dr
+    double* ang = cht + N;                                  // [N] angle 2 pi dr / N of receiver offset dr
+    unsigned long long* best = (unsigned long long*)(ang + N);   // [N] first-arrival key per dr
     float* qq = (float*)(best + N);                         // [n]
     float* ll = qq + n;                                     // [n]
     int* kk = (int*)(ll + n);                               // [n]
@@ -95,6 +99,7 @@ __global__ void __launch_bounds__(256) k_link(GeoDev G, const float* __restrict_
         sincos(two_pi * (double)r / (double)N, &yr, &xr);
         xr *= G.R_d;
         yr *= G.R_d;
+        ang[dr] = two_pi * (double)dr / (double)N;
         cht[dr] = sqrt((xr - xe) * (xr - xe) + (yr - ye) * (yr - ye)) / G.c_ref_d;
         if (F.n > 0) crs[dr] = bilinear_c(G, c, (float)xr, (float)yr);
         best[dr] = ~0ull;
@@ -112,7 +117,7 @@ __global__ void __launch_bounds__(256) k_link(GeoDev G, const float* __restrict_
             // receiver offsets whose angle 2 pi dr / N can lie in [lo, hi] (one spare each side)
             const int d0 = max(0, (int)floor(lo * dN) - 1), d1 = min(N - 1, (int)ceil(hi * dN) + 1);
             for (int dr = d0; dr <= d1; ++dr) {
-                const double thr = two_pi * (double)dr / (double)N;
+                const double thr = ang[dr];
                 if (thr < lo || thr > hi) continue;
                 double lam;
                 const unsigned long long key = d2key(bracket_T(cht[dr], a, b, thr, tr[i], tr[i + 1], &lam));
@@ -132,7 +137,7 @@ __global__ void __launch_bounds__(256) k_link(GeoDev G, const float* __restrict_
             for (int w = 0; w < F.n; ++w) p_out[(size_t)w * N * N + o] = make_float2(0.f, 0.f);
             continue;
         }
-        const double thr = two_pi * (double)dr / (double)N;
+        const double thr = ang[dr];
         double bestLam;
         const double bestT = bracket_T(cht[dr], th[bsel], th[bsel + 1], thr, tr[bsel], tr[bsel + 1], &bestLam);
         if (lrec) lrec[o] = LinkRec{bestT, bsel, (float)bestLam};
@@ -396,7 +401,7 @@ __global__ void k_sel_write(int n_total, const uint64_t* __restrict__ keys, cons
 cudaError_t launch_link(const GeoDev& G, const float* c, const rb_ray_end* ends, const FreqSet& F, float2* p_out,
                         uint8_t* linked, cudaStream_t s, LinkRec* lrec) {
     if (G.n_rays > LINK_MAX_RAYS) return cudaErrorInvalidValue;
-    const size_t sm = (size_t)G.n_rays * (8 + 8 + 4 + 4 + 4 + 4) + (size_t)G.n_elem * (8 + 8 + 4 + 4);
+    const size_t sm = (size_t)G.n_rays * (8 + 8 + 4 + 4 + 4 + 4) + (size_t)G.n_elem * (8 + 8 + 8 + 4 + 4);
     if (sm > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(k_link, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
         if (e != cudaSuccess) return e;
