@@ -227,13 +227,13 @@ __global__ void __launch_bounds__(256) k_tables_images(GeoDev G, const rb_cell* 
     const int e0 = 16 * eb + 8 * half;
     float4 sr[8];
     if (px < G.npix) {
-        const float c_px = __ldg(c + px);
+        const float sqrt_c = sqrtf(__ldg(c + px));
         const int ix = px % G.nx, iy = px / G.nx;
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
             DF ex, ey;
             elem_pos(G, e0 + k, ex, ey);
-            sr[k] = synth_record(tables[(size_t)(e0 + k) * G.npix + px], c_px, pixel_elem_dist(G, ix, iy, ex, ey),
+            sr[k] = synth_record(tables[(size_t)(e0 + k) * G.npix + px], sqrt_c, pixel_elem_dist(G, ix, iy, ex, ey),
                                  G.inv_cref, G.inv_cref_lo, G.j_floor);
         }
     } else {

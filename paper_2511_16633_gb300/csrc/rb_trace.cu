@@ -757,7 +757,7 @@ __global__ void __launch_bounds__(256) k_resolve_images(GeoDev G, const Vtx* __r
     const DF Y = df_pixel_coord(iy, G.cyg, G.h_hi, G.h_lo);
     const long long jx = 2LL * ix - (G.nx - 1), jy = 2LL * iy - (G.ny - 1);
     const bool in_support = live && jx * jx + jy * jy <= G.r2max;
-    const float c_px = live ? __ldg(c + pix) : 0.f;
+    const float sqrt_c = live ? sqrtf(__ldg(c + pix)) : 0.f;
     unsigned long long key[8];
 #pragma unroll
     for (int k = 0; k < 8; ++k) key[k] = live ? keys[(size_t)(e0 + k) * G.npix + pix] : ~0ull;
@@ -770,13 +770,12 @@ __global__ void __launch_bounds__(256) k_resolve_images(GeoDev G, const Vtx* __r
             const int e = e0 + 4 * kg + q;
             rb_cell rec;
             if (!resolve_entry(G, verts, ends, key[4 * kg + q], e, X, Y, kq_magic, rec)) {
-                sr[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+                rec = rb_cell{RB_HOLE, RB_HOLE, 0.f, 0.f};
                 if (in_support) ++holes;
-                continue;
             }
             DF ex, ey;
             elem_pos(G, e, ex, ey);
-            sr[q] = synth_record(rec, c_px, pixel_elem_dist(G, ix, iy, ex, ey), G.inv_cref, G.inv_cref_lo, G.j_floor);
+            sr[q] = synth_record(rec, sqrt_c, pixel_elem_dist(G, ix, iy, ex, ey), G.inv_cref, G.inv_cref_lo, G.j_floor);
         }
         for (int fw = 0; fw < F.n; ++fw) {
             __nv_bfloat16* plane = aimg + (size_t)fw * a_stride + (size_t)tile * 2 * rcn * 1024;
