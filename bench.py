@@ -120,16 +120,25 @@ def algorithmic_work(cfg, n_freq):
     return dict(adjoint_flop=adj_flop, forward_flop=fwd_flop, trace_grid_bytes=table_bytes)
 
 
-# Tensor FLOPs the BF16 x3 path issues per algorithmic FLOP: the gradient contraction
-# (8 n^2 npix per frequency) takes three bf16 products (hi.hi, hi.lo, lo.hi), the Hessian
-# contraction (2 n^2 npix) two (W is exact in bf16): (3 x 8 + 2 x 2) / (8 + 2).
-ADJ_ISSUE_RATIO = 2.8
+def adjoint_issue_ratio(n):
+    """Tensor FLOPs the BF16 x3 adjoint issues per algorithmic FLOP (10 n^2 npix per frequency).
+    Three bf16 products for the gradient, two for the Hessian diagonal (its weights are exact
+    in bf16), and of both symmetric sums only the blocks on and below the diagonal: K slices of
+    8 elements against 2 ne - 16 d columns, of 32 elements against ne - 32 d, in passes of ne
+    elements."""
+    ne = min(n, 256)
+    ge, gv = ne // 8, ne // 32
+    u = sum(16 * (2 * ne - 16 * max(0, j - q * ge)) for q in range(n // ne) for j in range((q + 1) * ge))
+    v = sum(32 * (ne - 32 * max(0, i - q * gv)) for q in range(n // ne) for i in range((q + 1) * gv))
+    return (3 * 2 * u + 2 * 2 * v) / (10.0 * n * n)
+
+
 # dram__bytes_read.sum + dram__bytes_write.sum of one k_adjoint_tc launch on breast512 from
 # one ncu capture (--metrics, one pass) of the kernel as it stands in ADJ_TRAFFIC_SOURCE;
 # set to None whenever the kernel changes until it is captured again.
-ADJ_TRAFFIC_BYTES = 2157880064 + 1073678080
+ADJ_TRAFFIC_BYTES = None
 ADJ_TRAFFIC_SOURCE = ("ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum, one k_adjoint_tc launch on "
-                      "breast512, kernel as of commit e24a358 (profiles/launches_breast512_bf16x3.md)")
+                      "breast512 (profiles/launches_breast512_bf16x3.md)")
 
 
 def rays_grid_bytes(cfg, n_vertices):
@@ -305,11 +314,11 @@ def run_ours(args):
               "updates_per_s": o["value"],
               "ms_per_update": o["ms_per_step"], "stage_ms": o["stage_ms"],
               "time_vs_one_step": o["ms_per_step"] / R["ms_per_step"],
-              # the gradient stages, 4 CG start kernels, per iteration a forward (+ reduce) and a
-              # B-image prep (mixed path) per frequency, one partial sum, the adjoint (+ its sum over
-              # the set's frequencies on the mixed path) and 3 vector kernels, then 3 apply/norm kernels
-              "gpu_launches_per_update": (20 + nf + args.cg_iters * (3 * nf + 6) if head == "bf16x3"
-                                          else 19 + args.cg_iters * (2 * nf + 5))}
+              # the gradient stages, 3 CG start kernels, per iteration a forward (+ reduce; plain path
+              # also G) per frequency, one partial sum, the operand prep, the adjoint (+ its sum over
+              # the set's frequencies on the mixed path) and 3 vector kernels, then 2 apply/norm kernels
+              "gpu_launches_per_update": (18 + args.cg_iters * (2 * nf + 7) if head == "bf16x3"
+                                          else 17 + args.cg_iters * (3 * nf + 6))}
     peaks, peak_src = _peaks()
     work = algorithmic_work(cfg, nf)
     st = R["stage_ms"]
@@ -333,15 +342,12 @@ def run_ours(args):
                 "peak_source": "derived: 152 SM x 128 FP32 lanes x 2 x max SM clock"}
 
     tc = head == "bf16x3"
-    # forward: the kernels compute the column blocks on and above the block diagonal of the
-    # symmetric real-form product (for 2n = 512 and 256-wide blocks: 6 of 8 block pairs)
-    nbn = (2 * cfg.n_elem + 255) // 256
-    nb = 2 * cfg.n_elem // nbn
+    # forward: three products, row blocks of 128 with the columns from their diagonal on (for
+    # 2n = 512: 1280 of 4 x 512 columns)
     nmb = 2 * cfg.n_elem // 128
-    done = sum(nbn - (128 * i) // nb for i in range(nmb))
-    fwd_ratio = 3.0 * done / (nmb * nbn)
+    fwd_ratio = 3.0 * (nmb + 1) / (2.0 * nmb)
     roof_adj = contraction_roof("adjoint", work["adjoint_flop"], "k_adjoint_tc" if tc else "k_adjoint_simt",
-                                ADJ_ISSUE_RATIO)
+                                adjoint_issue_ratio(cfg.n_elem))
     roof_fwd = contraction_roof("forward", work["forward_flop"], "k_forward_tc" if tc else "k_forward_simt", fwd_ratio)
     # the dominant kernel: the adjoint contraction (one launch per update, alone in its stage)
     roof = dict(roof_adj)
@@ -381,11 +387,12 @@ def run_ours(args):
         "roofline": roof, "roofline_contractions": {"adjoint": roof_adj, "forward": roof_fwd},
         "roofline_images": roof_img, "roofline_rays_grid": roof_rg,
         "clocks": R["clocks"], "e2e": R["e2e"],
-        # launches per update: positions, fields, keys reset, trace/raster/resolve (the resolve pass writes
-        # the operand images on the mixed path), link, residual keys and the three selection
-        # passes, adjoint (+ one B-image prep per frequency and the sum over the set's frequencies
-        # on the mixed path), 4 direction kernels, forward + reduce per frequency, 4 apply/norm kernels
-        "gpu_launches": (21 + 3 * nf) * args.steps if tc else (20 + 2 * nf) * args.steps,
+        # launches per update: fields, keys reset, trace/raster/resolve (the resolve pass writes the
+        # operand images on the mixed path), link, residual keys and the three selection passes,
+        # operand prep and adjoint (+ the sum over the set's frequencies on the mixed path), 2
+        # direction kernels, per frequency forward + reduce (plain path: G as well), 2 apply/norm
+        # kernels
+        "gpu_launches": (17 + 2 * nf) * args.steps if tc else (16 + 3 * nf) * args.steps,
         "diag_last": {k: R["diag"][k] for k in ("dc_norm", "alpha", "lost_rays", "holes", "kept", "zeroed")},
     }
     if tuned:

@@ -684,7 +684,9 @@ __device__ __forceinline__ bool resolve_entry(const GeoDev& G, const Vtx* __rest
 // Thread = pixel (its coordinates and support test computed once), looping over the
 // elements t = blockIdx.y, blockIdx.y + gridDim.y, ...; consecutive threads take
 // consecutive pixels, so every key load and record store is coalesced.
-// GREEN: the Green's functions of the set go out with the records, g[w][t][pixel].
+// GREEN: the Green's functions of the set go out with the records, g[w][t][pixel] (128
+// elements, 384 x 400 pixels, 2 frequencies: 386 us as two passes, 269 as one).  Holes keep
+// their early exit: without it more gathers are in flight, but the pass is slower.
 template <bool GREEN>
 __global__ void __launch_bounds__(256) k_resolve(GeoDev G, const Vtx* __restrict__ verts,
                                                  const rb_ray_end* __restrict__ ends,

@@ -7,8 +7,8 @@
 //
 // Every reduction is two-level with a fixed shape: a fixed grid writes one
 // double partial per block (fixed thread-to-element map, tree inside the
-// block) and a single block sums the partials in a fixed tree, so results do
-// not depend on scheduling.  All scalars stay on the device.
+// block) and whoever needs the scalar (one block, or every block of the next kernel) sums
+// the partials in a fixed tree, so results do not depend on scheduling.  All scalars stay on the device.
 #include "rb_internal.cuh"
 
 namespace {
