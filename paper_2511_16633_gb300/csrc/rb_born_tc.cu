@@ -928,12 +928,9 @@ __global__ void __launch_bounds__(NTHR_F, 1) k_forward_tc(const __grid_constant_
     const int nst = fwd_stages(cols);
     const int n_tiles = (G.npix + TP - 1) / TP;
     const int nsl_all = n_tiles * 8;
-    // Split sp takes slices sp, sp + S, ...: the splits are in proportion to what a slice costs,
-    // so every pair goes through the image at the same pace and what one has fetched the others
-    // find in L2.  (With a contiguous range per split the pairs, S apart, are at different places:
-    // the image was read twice, 1.08 GB a launch of 256 elements at 512 x 512 pixels, 187 us against
-    // 182; 511 x 389: 144 against 141.)
-    const int nq = sp < nsl_all ? (nsl_all - sp + S - 1) / S : 0;
+    const int cps = (nsl_all + S - 1) / S;
+    const int sbeg = min(nsl_all, sp * cps), send = min(nsl_all, sbeg + cps);
+    const int nq = send - sbeg;
     if (tid == 0) {
         for (int k = 0; k < nst; ++k) {
             tc::mbar_init(tc::smem_u32(&s_full_a[k]), 4);
@@ -964,7 +961,7 @@ __global__ void __launch_bounds__(NTHR_F, 1) k_forward_tc(const __grid_constant_
                 ok = false;
                 break;
             }
-            const int sg = sp + ql * S, x = (sg & 7) * 128, y0 = (sg >> 3) * 2 * rcn;
+            const int sg = sbeg + ql, x = (sg & 7) * 128, y0 = (sg >> 3) * 2 * rcn;
             const uint32_t mb = full_b0 + 8u * k, st = smem0 + (uint32_t)k * st_bytes;
             if (lead) {
                 tc::bulk_arm(mb, tx_bytes);
@@ -1042,7 +1039,7 @@ __global__ void __launch_bounds__(NTHR_F, 1) k_forward_tc(const __grid_constant_
         bool ok = true;
         auto load_m = [&](int q) -> float {
             if (q >= nq) return 0.f;
-            const int px = (sp + q * S) * 16 + pc * 8 + x8;
+            const int px = (sbeg + q) * 16 + pc * 8 + x8;
             return px < G.npix ? __ldg(A.m + px) : 0.f;
         };
         float mnext = load_m(grp);
