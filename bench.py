@@ -136,7 +136,7 @@ def adjoint_issue_ratio(n):
 # dram__bytes_read.sum + dram__bytes_write.sum of one k_adjoint_tc launch on breast512 from
 # one ncu capture (--metrics, one pass) of the kernel as it stands in ADJ_TRAFFIC_SOURCE;
 # set to None whenever the kernel changes until it is captured again.
-ADJ_TRAFFIC_BYTES = None
+ADJ_TRAFFIC_BYTES = 2150002944 + 469237248
 ADJ_TRAFFIC_SOURCE = ("ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum, one k_adjoint_tc launch on "
                       "breast512 (profiles/launches_breast512_bf16x3.md)")
 
