@@ -259,9 +259,11 @@ __global__ void __launch_bounds__(FTHR) k_forward_simt(GeoDev G, const float2* _
                     }
                 }
                 if (which == 0) {
+                    // a hole (G = 0) adds 0 whatever m holds there, which 0 x NaN or 0 x inf would not
                     const float mv = __ldg(m + pix);
-                    v.x *= mv;
-                    v.y *= mv;
+                    const bool any = v.x != 0.f || v.y != 0.f;
+                    v.x = any ? v.x * mv : 0.f;
+                    v.y = any ? v.y * mv : 0.f;
                 }
             }
             if (which == 0) Ae[p][tl] = v; else Br[p][tl] = v;
