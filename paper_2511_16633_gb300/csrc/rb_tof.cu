@@ -145,8 +145,8 @@ __global__ void __launch_bounds__(RT) k_tof_coef(GeoDev G, const LinkRec* __rest
     if (bm > 0.f) atomicMax(&amax[1], __float_as_uint(bm));
 }
 
-// A pixel's weight in a ray's path, in units of 2^-43 of the power of two at or above ds
-// (scale: 2^21 over it): exact for float weights down to 2^-19 of that, as a sum in double.
+// A pixel's weight in a ray's path, in units of 2^-52 of the power of two at or above ds
+// (scale: 2^30 over it), as fine as a sum in double: exact for float weights down to 2^-29 of it.
 __device__ __forceinline__ unsigned long long fix_weight(float w, float scale) {
     const float t = w * scale;
     const uint32_t hi = (uint32_t)t;
@@ -154,11 +154,12 @@ __device__ __forceinline__ unsigned long long fix_weight(float w, float scale) {
     return ((unsigned long long)hi << 22) + lo;
 }
 
-// A coefficient (units of the largest one / 2^52) times a weight, into a pixel sum in units
-// of the largest coefficient x that power of two / 2^40, rounded to one unit.
+// A coefficient (in units of the largest one times ds over that power of two, / 2^52) times a
+// weight, into a pixel sum in units of the largest coefficient x ds / 2^40, rounded to one unit:
+// the product over 2^64.  |a| <= 2^53 and a piece's weights are 64 x 2^52 at most.
 __device__ __forceinline__ void deposit(unsigned long long* __restrict__ dst, long long a, unsigned long long w) {
-    const long long x = a * (1LL << 9), y = (long long)w;   // a w / 2^55 = the product's high half
-    const long long q = __mul64hi(x, y) + (long long)(((unsigned long long)x * (unsigned long long)y) >> 63);
+    const long long y = (long long)w;
+    const long long q = __mul64hi(a, y) + (long long)(((unsigned long long)a * w) >> 63);
     if (q != 0) atomicAdd(dst, (unsigned long long)q);
 }
 
@@ -170,15 +171,15 @@ __device__ __forceinline__ void deposit(unsigned long long* __restrict__ dst, lo
 // 1774 us, most of it on the FP64 pipe (2 lanes a cycle and SM); 460 us so.
 __global__ void __launch_bounds__(128) k_tof_bp(GeoDev G, const Vtx* __restrict__ verts, const rb_ray_end* __restrict__ ends,
                                                 int n_pieces, const float2* __restrict__ coef,
-                                                const uint32_t* __restrict__ amax, float wscale,
+                                                const uint32_t* __restrict__ amax, float wscale, double cscale,
                                                 unsigned long long* __restrict__ num, unsigned long long* __restrict__ den) {
     TofPiece w;
     if (!tof_piece(G, ends, n_pieces, &w)) return;
     const float2 cf = coef[(size_t)w.t * G.n_rays + w.i];
     if (cf.x == 0.f && cf.y == 0.f) return;
     const float am = __uint_as_float(amax[0]), bm = __uint_as_float(amax[1]);
-    const long long ca = am > 0.f ? __double2ll_rn((double)cf.x / (double)am * 4503599627370496.0) : 0;
-    const long long cb = bm > 0.f ? __double2ll_rn((double)cf.y / (double)bm * 4503599627370496.0) : 0;
+    const long long ca = am > 0.f ? __double2ll_rn((double)cf.x / (double)am * cscale) : 0;
+    const long long cb = bm > 0.f ? __double2ll_rn((double)cf.y / (double)bm * cscale) : 0;
     unsigned long long w00 = 0, w10 = 0, w01 = 0, w11 = 0;
     int qi = -1, qj = -1;
     auto put = [&](int di, int dj, unsigned long long& wt) {
@@ -256,7 +257,7 @@ __global__ void __launch_bounds__(RT) k_tof_apply(GeoDev G, float* __restrict__ 
     for (int p = blockIdx.x * RT + threadIdx.x; p < G.npix; p += gridDim.x * RT) {
         const long long dq = (long long)den[p];
         if (dq <= 0 || !in_support_px(G, p)) continue;
-        // num / den back in physical units: (nq am u / 2^40) / (dq bm u / 2^40), u the power of two above ds
+        // num / den back in physical units: (nq am ds / 2^40) / (dq bm ds / 2^40)
         const double ds = ((double)(long long)num[p] * (double)am) / ((double)dq * (double)bm);
         c[p] = (float)(1.0 / (1.0 / (double)c[p] + ds));
     }
@@ -387,8 +388,9 @@ cudaError_t launch_tof_step(const GeoDev& G, const Vtx* verts, const rb_ray_end*
     }
     k_tof_coef<<<G.n_elem, RT, sm, s>>>(G, w.lrec, t_obs, obs_linked, w.len, w.coef, w.amax);
     int ex = 0;
-    frexp(G.ds_d, &ex);   // ds < 2^ex
-    k_tof_bp<<<rb, 128, 0, s>>>(G, verts, ends, n_pieces, w.coef, w.amax, (float)ldexp(1.0, 21 - ex), w.num, w.den);
+    const double mant = frexp(G.ds_d, &ex);   // ds = mant 2^ex, mant in [0.5, 1)
+    k_tof_bp<<<rb, 128, 0, s>>>(G, verts, ends, n_pieces, w.coef, w.amax, (float)ldexp(1.0, 30 - ex),
+                                4503599627370496.0 / mant, w.num, w.den);
     k_tof_apply<<<RB, RT, 0, s>>>(G, c, w.num, w.den, w.amax);
     return cudaGetLastError();
 }
