@@ -1131,13 +1131,26 @@ __global__ void __launch_bounds__(256) k_forward_tc_reduce(FwdArgs A, float2* __
             const int i = (2 * e) >> 7, row = (2 * e) & 127, pq = A.pidx[i][(2 * r) >> 9], ns = A.splits[pq];
             const float* blk = A.partial + ((size_t)A.cta0[pq] * 128 + row) * n2 + 2 * r;
             const size_t step = (size_t)128 * n2;
-#pragma unroll 8
-            for (int sp = y; sp < ns; sp += YS) {
-                const float2 a0 = *(const float2*)(blk + sp * step), a1 = *(const float2*)(blk + sp * step + n2);
-                s.x += a0.x;
-                s.y += a0.y;
-                s.z += a1.x;
-                s.w += a1.y;
+            // eight splits ahead: a split's loads go out as the one eight before it is added
+            float2 n0[8], n1[8];
+            auto load = [&](int k, int sp) {
+                n0[k] = n1[k] = make_float2(0.f, 0.f);
+                if (sp < ns) {
+                    n0[k] = __ldcg((const float2*)(blk + sp * step));
+                    n1[k] = __ldcg((const float2*)(blk + sp * step + n2));
+                }
+            };
+#pragma unroll
+            for (int k = 0; k < 8; ++k) load(k, y + k * YS);
+            for (int sp = y; sp < ns; sp += 8 * YS) {
+#pragma unroll
+                for (int k = 0; k < 8; ++k) {
+                    s.x += n0[k].x;
+                    s.y += n0[k].y;
+                    s.z += n1[k].x;
+                    s.w += n1[k].y;
+                    load(k, sp + (8 + k) * YS);
+                }
             }
         }
         if (YS > 1) {
