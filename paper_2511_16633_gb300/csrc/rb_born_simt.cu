@@ -8,7 +8,8 @@
 // diagonal blocks.  One CTA owns a tile of 32 pixels: it synthesises G_t(x) for every
 // element and the tile's pixels into shared memory (Eqs. 4-5), runs both contractions with
 // T and Y streamed through shared memory, and reduces over e in a fixed order, so g and H
-// never need U or V in HBM and every pixel's result is independent of scheduling.
+// never need U or V in HBM and every pixel's result is independent of scheduling.  Rings below
+// 48 elements take the full sums over r instead (k_adjoint_small).
 //
 // Forward: d[e][r] = w^2 sum_x G_e(x) G_r(x) m(x), symmetric in (e, r).  G of the frequency is
 // synthesised once into a buffer; split-K over pixel chunks: CTA (tile pair, chunk)
@@ -73,6 +74,47 @@ __global__ void __launch_bounds__(256) k_prep_sym(int n, int nb, const float2* _
 
 __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
+
+// The 32 parts of g and H of a tile's pixels (part q of this thread's pixels 4 tx .. 4 tx + 3),
+// added in order by the pixels' threads, out, and into their sums over the set.
+__device__ __forceinline__ void sum_parts(const GeoDev& G, const FreqC& fc, int fw, int p0, int tx, int q, const float pg_r[4],
+                                          const float pg_i[4], const float ph[4], float* red, float2* __restrict__ g_out,
+                                          float* __restrict__ h_out, float& acc_g, float& acc_h) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const int p = tx * 4 + j;
+        red[(q * AP + p) * 3 + 0] = pg_r[j];
+        red[(q * AP + p) * 3 + 1] = pg_i[j];
+        red[(q * AP + p) * 3 + 2] = ph[j];
+    }
+    __syncthreads();
+    if (threadIdx.x < AP) {
+        const int p = threadIdx.x;
+        float sr = 0.f, si = 0.f, sh = 0.f;
+        for (int k = 0; k < 32; ++k) {
+            sr += red[(k * AP + p) * 3 + 0];
+            si += red[(k * AP + p) * 3 + 1];
+            sh += red[(k * AP + p) * 3 + 2];
+        }
+        sr *= fc.w2;
+        si *= fc.w2;
+        sh *= fc.w4;
+        const int pix = p0 + p;
+        if (pix < G.npix) {
+            if (g_out) g_out[(size_t)fw * G.npix + pix] = make_float2(sr, si);
+            if (h_out) h_out[(size_t)fw * G.npix + pix] = sh;
+        }
+        acc_g += sr;
+        acc_h += sh;
+    }
+}
+__device__ __forceinline__ void store_sums(const GeoDev& G, int p0, float acc_g, float acc_h, float* __restrict__ gsum,
+                                           float* __restrict__ hsum) {
+    const int pix = p0 + (int)threadIdx.x;
+    if (threadIdx.x >= AP || pix >= G.npix) return;
+    if (gsum) gsum[pix] = acc_g;
+    if (hsum) hsum[pix] = acc_h;
 }
 
 // Chunks of 32 r x 32 e (16 KB) go through two shared-memory buffers (cp.async); of each
@@ -163,41 +205,92 @@ __global__ void __launch_bounds__(AT, 2) k_adjoint_simt(GeoDev G, const rb_cell*
             rb = rb1;
         }
         __syncthreads();   // every thread is done with the buffers that red reuses
+        sum_parts(G, fc, fw, p0, tx, tz * 8 + ty, pg_r, pg_i, ph, red, g_out, h_out, acc_g, acc_h);
+    }
+    store_sums(G, p0, acc_g, acc_h, gsum, hsum);
+}
+
+// The full sums over r, for the rings whose padding to blocks of 32 would cost more than the
+// symmetric sums save: S and W go through shared memory eight r at a time, and a thread
+// accumulates the elements ty + 32 i, i < EPT, at 4 pixels.
+constexpr int RC = 8;        // r-chunk of S / W staged in shared memory
+constexpr int RCP = RC + 1;  // padded row (conflict-free reads by the 4 element rows of a warp)
+template <int EPT>
+__global__ void __launch_bounds__(AT) k_adjoint_small(GeoDev G, const rb_cell* __restrict__ tables, const float* __restrict__ c,
+                                                      FreqSet F, const float2* __restrict__ resid, const uint8_t* __restrict__ w,
+                                                      float2* __restrict__ g_out, float* __restrict__ h_out,
+                                                      float* __restrict__ gsum, float* __restrict__ hsum) {
+    extern __shared__ float4 smem4[];
+    const int n = G.n_elem;
+    float2* Gs = (float2*)smem4;                 // [n][AP]
+    float2* Ss = Gs + (size_t)n * AP;            // [n][RCP]
+    float* Ws = (float*)(Ss + (size_t)n * RCP);  // [n][RCP]
+    float* red = (float*)Ss;                     // [32][AP][3], reuses the S / W staging after the r loop
+    const int tx = threadIdx.x & 7, ty = threadIdx.x >> 3;   // pixels tx*4 .. tx*4+3
+    const int p0 = blockIdx.x * AP;
+    float acc_g = 0.f, acc_h = 0.f;
+    for (int fw = 0; fw < F.n; ++fw) {
+        const FreqC& fc = F.f[fw];
+        const float2* Rw = resid + (size_t)fw * n * n;
+        const uint8_t* Ww = w + (size_t)fw * n * n;
+        __syncthreads();   // the previous frequency's sums are out of the staging
+        synth_tile(G, tables, c, fc, p0, n, Gs);
+        float ur[EPT][4], ui[EPT][4], vv[EPT][4];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int p = tx * 4 + j, q = tz * 8 + ty;
-            red[(q * AP + p) * 3 + 0] = pg_r[j];
-            red[(q * AP + p) * 3 + 1] = pg_i[j];
-            red[(q * AP + p) * 3 + 2] = ph[j];
-        }
-        __syncthreads();
-        if (threadIdx.x < AP) {
-            const int p = threadIdx.x;
-            float sr = 0.f, si = 0.f, sh = 0.f;
-            for (int q = 0; q < 32; ++q) {
-                sr += red[(q * AP + p) * 3 + 0];
-                si += red[(q * AP + p) * 3 + 1];
-                sh += red[(q * AP + p) * 3 + 2];
+        for (int i = 0; i < EPT; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) ur[i][j] = ui[i][j] = vv[i][j] = 0.f;
+        for (int r0 = 0; r0 < n; r0 += RC) {
+            __syncthreads();
+            for (int idx = threadIdx.x; idx < n * RC; idx += blockDim.x) {
+                const int e = idx / RC, rr = idx % RC, r = r0 + rr;
+                const bool used = r < n && Ww[(size_t)e * n + r];
+                Ss[e * RCP + rr] = used ? Rw[(size_t)e * n + r] : make_float2(0.f, 0.f);
+                Ws[e * RCP + rr] = used ? 1.f : 0.f;
             }
-            sr *= fc.w2;
-            si *= fc.w2;
-            sh *= fc.w4;
-            const int pix = p0 + p;
-            if (pix < G.npix) {
-                if (g_out) g_out[(size_t)fw * G.npix + pix] = make_float2(sr, si);
-                if (h_out) h_out[(size_t)fw * G.npix + pix] = sh;
+            __syncthreads();
+            const int rmax = min(RC, n - r0);
+            for (int rr = 0; rr < rmax; ++rr) {
+                const float4* gp = (const float4*)(Gs + (size_t)(r0 + rr) * AP + tx * 4);
+                const float4 g01 = gp[0], g23 = gp[1];
+                const float br[4] = {g01.x, g01.z, g23.x, g23.z};
+                const float bi[4] = {-g01.y, -g01.w, -g23.y, -g23.w};   // conj(G_r)
+                float a2[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) a2[j] = br[j] * br[j] + bi[j] * bi[j];
+#pragma unroll
+                for (int i = 0; i < EPT; ++i) {
+                    const int e = ty + 32 * i;
+                    const float2 s = e < n ? Ss[e * RCP + rr] : make_float2(0.f, 0.f);
+                    const float wv = e < n ? Ws[e * RCP + rr] : 0.f;
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        ur[i][j] = fmaf(s.x, br[j], fmaf(-s.y, bi[j], ur[i][j]));
+                        ui[i][j] = fmaf(s.x, bi[j], fmaf(s.y, br[j], ui[i][j]));
+                        vv[i][j] = fmaf(wv, a2[j], vv[i][j]);
+                    }
+                }
             }
-            acc_g += sr;
-            acc_h += sh;
         }
-    }
-    if (threadIdx.x < AP) {
-        const int pix = p0 + threadIdx.x;
-        if (pix < G.npix) {
-            if (gsum) gsum[pix] = acc_g;
-            if (hsum) hsum[pix] = acc_h;
+        float pg_r[4], pg_i[4], ph[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) pg_r[j] = pg_i[j] = ph[j] = 0.f;
+#pragma unroll
+        for (int i = 0; i < EPT; ++i) {
+            const int e = ty + 32 * i;
+            if (e >= n) continue;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const float2 ge = Gs[(size_t)e * AP + tx * 4 + j];
+                pg_r[j] += ge.x * ur[i][j] + ge.y * ui[i][j];   // conj(G_e) U
+                pg_i[j] += ge.x * ui[i][j] - ge.y * ur[i][j];
+                ph[j] += (ge.x * ge.x + ge.y * ge.y) * vv[i][j];
+            }
         }
+        __syncthreads();   // every thread is done with the staging that red reuses
+        sum_parts(G, fc, fw, p0, tx, ty, pg_r, pg_i, ph, red, g_out, h_out, acc_g, acc_h);
     }
+    store_sums(G, p0, acc_g, acc_h, gsum, hsum);
 }
 
 // ---------------------------------------------------------------------------
@@ -383,13 +476,26 @@ cudaError_t launch_adjoint_simt(const GeoDev& G, const rb_cell* tables, const fl
                                 float* hsum, void* sym, cudaStream_t s) {
     if (!simt_adjoint_supported(G.n_elem)) return cudaErrorInvalidValue;
     const int n = G.n_elem, nb = (n + EB - 1) / EB;
+    const int blocks = (G.npix + AP - 1) / AP;
+    // Rings below 48 elements take the full sums.  Measured at 512 x 500 pixels, symmetric against
+    // full: 8 elements 134 and 59 us, 20: 178 and 123, 32: 203 and 179, 33: 330 and 261, 44: 360
+    // and 343, 48: 363 and 368, 60: 403 and 473; at 64 x 64 pixels, 8 elements: 17 and 13 (the
+    // operand's own launch).
+    if (n < 48) {
+        size_t stage = (size_t)n * RCP * (sizeof(float2) + sizeof(float));
+        if (stage < (size_t)32 * AP * 3 * sizeof(float)) stage = (size_t)32 * AP * 3 * sizeof(float);
+        const size_t sm = (size_t)n * AP * sizeof(float2) + stage;   // 29 KB at most
+        if (n <= 32) k_adjoint_small<1><<<blocks, AT, sm, s>>>(G, tables, c, F, resid, w, g_out, h_out, gsum, hsum);
+        else k_adjoint_small<2><<<blocks, AT, sm, s>>>(G, tables, c, F, resid, w, g_out, h_out, gsum, hsum);
+        return cudaGetLastError();
+    }
     k_prep_sym<<<dim3(nb, F.n, 8), 256, 0, s>>>(n, nb, resid, w, (float4*)sym);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     const size_t sm = (size_t)2 * EB * EB * sizeof(float4) + (size_t)nb * EB * AP * sizeof(float2);
     e = cudaFuncSetAttribute(k_adjoint_simt, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
-    k_adjoint_simt<<<(G.npix + AP - 1) / AP, AT, sm, s>>>(G, tables, c, F, (const float4*)sym, g_out, h_out, gsum, hsum);
+    k_adjoint_simt<<<blocks, AT, sm, s>>>(G, tables, c, F, (const float4*)sym, g_out, h_out, gsum, hsum);
     return cudaGetLastError();
 }
 
