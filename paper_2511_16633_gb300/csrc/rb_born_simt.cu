@@ -297,9 +297,14 @@ __global__ void __launch_bounds__(AT) k_adjoint_small(GeoDev G, const rb_cell* _
 // Forward
 // ---------------------------------------------------------------------------
 constexpr int FT = 64;      // element tile
-constexpr int FP = 16;      // pixels per sub-tile
 constexpr int FS = FT + 2;  // padded row of a sub-tile (16-byte aligned)
-constexpr int FTHR = 128;   // 8 x 16 threads, 8 x 4 complex outputs each
+// Threads of a forward CTA (64 rows over threads / 16 of them: 8 or 4 x 4 complex outputs a thread)
+// and pixels per sub-tile.  Where the CTAs synthesise G, half their time goes by waiting for its
+// special functions, and the scratch of a call without a workspace holds too few chunks for more
+// than one or two CTAs an SM: twice the threads each (256 elements, 256 x 256 pixels: 2320 us,
+// 3340 with 128 threads; 1000 elements, 128 x 120: 6817 and 10887; 64 elements, 64 x 64: 33 and 42).
+constexpr int fwd_threads(bool from_g) { return from_g ? 128 : 256; }
+constexpr int fwd_pixels(bool from_g) { return from_g ? 16 : 32; }
 
 // FROM_G: G of the frequency comes from the buffer g [n_elem][npix]; otherwise (no workspace)
 // it is synthesised from the tables, once per tile pair that uses it.  Bound by the FP32
@@ -307,9 +312,10 @@ constexpr int FTHR = 128;   // 8 x 16 threads, 8 x 4 complex outputs each
 // pixels: 416 us and 72 for G (1189 us with a 4 x 4 tile a thread and G synthesised for every
 // pair, half the time the synthesis).
 template <bool FROM_G>
-__global__ void __launch_bounds__(FTHR) k_forward_simt(GeoDev G, const float2* __restrict__ g, const rb_cell* __restrict__ tables,
+__global__ void __launch_bounds__(fwd_threads(FROM_G)) k_forward_simt(GeoDev G, const float2* __restrict__ g, const rb_cell* __restrict__ tables,
                                                        const float* __restrict__ c, FreqC F, const float* __restrict__ m,
                                                        float2* __restrict__ partial, int n_chunks) {
+    constexpr int FTHR = fwd_threads(FROM_G), FP = fwd_pixels(FROM_G), ER = FT * 16 / FTHR;   // rows e a thread
     __shared__ __align__(16) float2 Ae[FP][FS];   // G_e(x) m(x), transposed [p][e]
     __shared__ __align__(16) float2 Br[FP][FS];   // G_r(x)
     const int n = G.n_elem;
@@ -323,9 +329,9 @@ __global__ void __launch_bounds__(FTHR) k_forward_simt(GeoDev G, const float2* _
     const int pbeg = min(G.npix, chunk * pix_per), pend = min(G.npix, pbeg + pix_per);
     const int e0 = te * FT, r0 = tr * FT;
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    float ar[8][4], ai[8][4];
+    float ar[ER][4], ai[ER][4];
 #pragma unroll
-    for (int i = 0; i < 8; ++i)
+    for (int i = 0; i < ER; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j) ar[i][j] = ai[i][j] = 0.f;
 
@@ -365,14 +371,14 @@ __global__ void __launch_bounds__(FTHR) k_forward_simt(GeoDev G, const float2* _
         const int np = min(FP, pend - ps);
 #pragma unroll 2
         for (int p = 0; p < np; ++p) {
-            float4 a4[4], b4[2];
+            float4 a4[ER / 2], b4[2];
 #pragma unroll
-            for (int i = 0; i < 4; ++i) a4[i] = *(const float4*)&Ae[p][ty * 8 + 2 * i];
+            for (int i = 0; i < ER / 2; ++i) a4[i] = *(const float4*)&Ae[p][ty * ER + 2 * i];
 #pragma unroll
             for (int i = 0; i < 2; ++i) b4[i] = *(const float4*)&Br[p][tx * 4 + 2 * i];
             const float bx[4] = {b4[0].x, b4[0].z, b4[1].x, b4[1].z}, by[4] = {b4[0].y, b4[0].w, b4[1].y, b4[1].w};
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
+            for (int i = 0; i < ER; ++i) {
                 const float ax = (i & 1) ? a4[i >> 1].z : a4[i >> 1].x, ay = (i & 1) ? a4[i >> 1].w : a4[i >> 1].y;
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
@@ -385,10 +391,10 @@ __global__ void __launch_bounds__(FTHR) k_forward_simt(GeoDev G, const float2* _
     // partial[chunk][e][r] for this block (upper-triangle tile pairs only)
     float2* out = partial + (size_t)chunk * n * n;
 #pragma unroll
-    for (int i = 0; i < 8; ++i)
+    for (int i = 0; i < ER; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            const int e = e0 + ty * 8 + i, r = r0 + tx * 4 + j;
+            const int e = e0 + ty * ER + i, r = r0 + tx * 4 + j;
             if (e < n && r < n) out[(size_t)e * n + r] = make_float2(ar[i][j], ai[i][j]);
         }
 }
@@ -522,7 +528,7 @@ cudaError_t launch_forward_simt(const GeoDev& G, const rb_cell* tables, const fl
     const int nt = (G.n_elem + FT - 1) / FT;
     const dim3 grid(nt * (nt + 1) / 2, n_chunks);
     if (!g_buf) {
-        k_forward_simt<false><<<grid, FTHR, 0, s>>>(G, nullptr, tables, c, F, m, partial, n_chunks);
+        k_forward_simt<false><<<grid, fwd_threads(false), 0, s>>>(G, nullptr, tables, c, F, m, partial, n_chunks);
         return cudaGetLastError();
     }
     const int bx = (G.npix + 255) / 256;
@@ -531,7 +537,7 @@ cudaError_t launch_forward_simt(const GeoDev& G, const rb_cell* tables, const fl
     k_green_out<<<dim3(bx, by), 256, 0, s>>>(G, tables, c, F, g_buf);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    k_forward_simt<true><<<grid, FTHR, 0, s>>>(G, g_buf, tables, c, F, m, partial, n_chunks);
+    k_forward_simt<true><<<grid, fwd_threads(true), 0, s>>>(G, g_buf, tables, c, F, m, partial, n_chunks);
     return cudaGetLastError();
 }
 
