@@ -402,33 +402,50 @@ __global__ void __launch_bounds__(fwd_threads(FROM_G)) k_forward_simt(GeoDev G, 
 // d[e][r] = w^2 sum_chunk partial (fixed order), entries right of the diagonal tiles mirrored
 // into the lower triangle; optional sum of W |d|^2 into per-block partials.  A CTA takes 32
 // consecutive r of one e at a time; its 8 warps take every eighth chunk, warp 0 adds the
-// warps' sums in order.
+// warps' sums in order.  YS = 1, for up to eight chunks: a warp takes 32 entries by itself,
+// in the same order (1000 elements, 16 x 15 pixels, the whole forward in one chunk: 270 us by
+// eight warps with their barriers a run, 140 so).
+template <int YS>
 __global__ void __launch_bounds__(256) k_forward_reduce(GeoDev G, FreqC F, const float2* __restrict__ partial, int n_chunks,
                                                         float2* __restrict__ d_out, const uint8_t* __restrict__ w,
                                                         double* __restrict__ den_part) {
     __shared__ float2 s_sum[8][32];
-    const int n = G.n_elem, lane = threadIdx.x & 31, y = threadIdx.x >> 5, nrb = (n + 31) / 32;
+    __shared__ double s_den[8];
+    const int n = G.n_elem, lane = threadIdx.x & 31, wid = threadIdx.x >> 5, y = wid % YS, nrb = (n + 31) / 32;
     const size_t total = (size_t)n * n;
     double acc = 0.0;
-    for (int tile = blockIdx.x; tile < n * nrb; tile += gridDim.x) {
+    constexpr int TPB = 8 / YS;   // runs of 32 entries a CTA takes at a time
+    for (int tile0 = blockIdx.x * TPB; tile0 < n * nrb; tile0 += gridDim.x * TPB) {
+        const int tile = tile0 + wid / YS;
         const int e = tile / nrb, rb = tile - e * nrb, r = 32 * rb + lane;
         const int te = e / FT, tr = 32 * rb / FT;   // a 32-entry run lies in one tile
-        if (tr < te) continue;
+        if (e >= n || tr < te) continue;            // YS = 8: the whole CTA's run
         float sr = 0.f, si = 0.f;
         if (r < n) {
+            // eight chunks ahead: a chunk's load goes out as the one eight before it is added
             const float2* src = partial + (size_t)e * n + r;
-#pragma unroll 4
-            for (int ch = y; ch < n_chunks; ch += 8) {
-                const float2 v = src[(size_t)ch * total];
-                sr += v.x;
-                si += v.y;
+            float2 nx[8];
+            auto load = [&](int k, int ch) {
+                nx[k] = ch < n_chunks ? __ldcg(src + (size_t)ch * total) : make_float2(0.f, 0.f);
+            };
+#pragma unroll
+            for (int k = 0; k < 8; ++k) load(k, y + k * YS);
+            for (int ch = y; ch < n_chunks; ch += 8 * YS) {
+#pragma unroll
+                for (int k = 0; k < 8; ++k) {
+                    sr += nx[k].x;
+                    si += nx[k].y;
+                    load(k, ch + (8 + k) * YS);
+                }
             }
         }
-        __syncthreads();
-        s_sum[y][lane] = make_float2(sr, si);
-        __syncthreads();
+        if (YS > 1) {
+            __syncthreads();
+            s_sum[y][lane] = make_float2(sr, si);
+            __syncthreads();
+        }
         if (y == 0 && r < n) {
-            for (int k = 1; k < 8; ++k) {
+            for (int k = 1; k < YS; ++k) {
                 sr += s_sum[k][lane].x;
                 si += s_sum[k][lane].y;
             }
@@ -446,9 +463,14 @@ __global__ void __launch_bounds__(256) k_forward_reduce(GeoDev G, FreqC F, const
             }
         }
     }
-    if (den_part && y == 0) {
+    if (den_part) {
         for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
-        if (lane == 0) den_part[blockIdx.x] = acc;
+        if (lane == 0) s_den[wid] = acc;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            for (int k = 1; k < 8; ++k) acc += s_den[k];   // 0 from the warps that only helped
+            den_part[blockIdx.x] = acc;
+        }
     }
 }
 
@@ -543,6 +565,7 @@ cudaError_t launch_forward_simt(const GeoDev& G, const rb_cell* tables, const fl
 
 cudaError_t launch_forward_reduce(const GeoDev& G, const FreqC& F, const float2* partial, int n_chunks, float2* d_out,
                                   const uint8_t* w, double* den_part, cudaStream_t s) {
-    k_forward_reduce<<<256, 256, 0, s>>>(G, F, partial, n_chunks, d_out, w, den_part);
+    if (n_chunks <= 8) k_forward_reduce<1><<<256, 256, 0, s>>>(G, F, partial, n_chunks, d_out, w, den_part);
+    else k_forward_reduce<8><<<256, 256, 0, s>>>(G, F, partial, n_chunks, d_out, w, den_part);
     return cudaGetLastError();
 }

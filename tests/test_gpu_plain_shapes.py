@@ -1,6 +1,7 @@
 """The plain FP32 operators at the sizes where their kernels change: rings below 48 elements, whose
-adjoint multiplies out the full sums (one or two elements a thread, chunks of eight r).
-References and tolerances as in test_gpu_born_shapes.py (FP32 sums against 64 bits: 1e-5 relative L2)."""
+adjoint multiplies out the full sums (one or two elements a thread, chunks of eight r), and
+forwards of few pixel chunks, which a warp sums by itself.  References and tolerances as in
+test_gpu_born_shapes.py (FP32 sums against 64 bits: 1e-5 relative L2)."""
 import math
 
 import pytest
@@ -30,3 +31,19 @@ def test_adjoint_of_small_rings(dev, n, nx, ny):  # noqa: F811
         assert _rel(out, w2 * (G.conj() * (Sw @ G.conj())).sum(0)) <= 1e-5
         if want_h:
             assert _rel(h, w2 * w2 * (P * (W.double() @ P)).sum(0)) <= 1e-5
+
+
+# two chunks (the smallest grid that a ring fits), eight, ten, and the fixed scratch's single chunk
+# for a thousand elements
+@pytest.mark.parametrize("n,nx,ny", [(70, 6, 6), (33, 16, 16), (70, 17, 17), (600, 16, 15), (1000, 12, 11)])
+def test_forward_of_few_chunks(dev, n, nx, ny):  # noqa: F811
+    geom, tab, c, G, f, g = _problem(dev, n, nx, ny)
+    m = 1e-9 * torch.randn(nx * ny, generator=g, device=dev)
+    ref = (2 * math.pi * f) ** 2 * (G * m.double()) @ G.T
+    ws = rb.workspace(geom, 1, rb.RB_PREC_FP32, dev)
+    d = torch.full((n, n), float("nan"), dtype=torch.complex64, device=dev)
+    rb.rb_born_forward(geom, tab, c, f, m, d, ws, rb.RB_PREC_FP32)
+    assert _rel(d, ref) <= 1e-5
+    d.fill_(float("nan"))
+    rb.rb_born_forward_noalloc(geom, tab, c, f, m, d)
+    assert _rel(d, ref) <= 1e-5
