@@ -510,8 +510,7 @@ def main():
     ap.add_argument("--tune", default="on",
                     help="on: run with the kernel-shape choice the tuner measures fastest on this problem (tuned "
                          "before the warm-up); off: the library's rule; an integer: that kernel-shape code "
-                         "(rb_update_params.tune: 1 raster along tubes, 2 across; + 4 adjoint CTA pairs, + 8 one CTA "
-                         "per tile)")
+                         "(rb_update_params.tune: 1 raster along tubes, 2 across; + 4 or + 8 accepted, one form)")
     ap.add_argument("--cg-iters", type=int, default=12,
                     help="also time the CG variant of the update with this many iterations (0: skip)")
     args = ap.parse_args()

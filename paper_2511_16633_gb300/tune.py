@@ -3,9 +3,10 @@
 The rasteriser of the gridding has two work mappings, warps along the ray tubes or
 across them, whose speed depends on how wide the tubes are against the pixels and on
 how much the medium bends them; the library's rule picks by tube width alone.  The
-tensor-core adjoint has one form, one CTA per pixel tile; the field that chose CTA pairs
-before is still accepted, and its values are still told apart here.  The choices do not change the results, so only their time differs, and that is
-measured here: for one problem, ``tune_update`` times the updates per candidate on
+tensor-core adjoint has one form, one CTA per pixel tile: the codes of the field that
+chose CTA pairs before are accepted and reported, and run that form.  The choices do not
+change the results, so only their time differs, and that is measured here: for one
+problem, ``tune_update`` times the updates once per form that differs (``forms``) on
 the caller's own data (a warm-up run, then ``reps`` timed ones, each from a scratch
 copy of c, with CUDA events on a private stream; a whole sweep over the problem's
 frequency sets when they are given), keeps the fastest and caches it per key (ring,
@@ -25,11 +26,16 @@ ADJOINT = {rb.RB_TUNE_ADJ_SINGLE: "adjoint one CTA per tile", rb.RB_TUNE_ADJ_PAI
 
 
 def candidates(prec: int):
-    """The tune values tried for a precision: both raster mappings, and on the tensor-core
-    path both values of the adjoint's field."""
+    """The tune values accepted for a precision: both raster mappings, and on the tensor-core
+    path both values of the adjoint's field, which mean the same kernel."""
     if prec == rb.RB_PREC_BF16X3:
         return tuple(r | a for a in ADJOINT for r in RASTER)
     return tuple(RASTER)
+
+
+def forms(prec: int):
+    """One tune value for each form that differs: the raster mappings."""
+    return tuple(c for c in candidates(prec) if not c & rb.RB_TUNE_ADJ_PAIR)
 
 
 def name(tune: int) -> str:
@@ -83,8 +89,8 @@ def cached(geom, n_freq: int, prec: int) -> Optional[dict]:
 
 
 def tune_update(geom, c, alpha0, freqs, p_obs, prec, reps: int = 3, device=None, sets=None) -> Tuple[int, dict]:
-    """The fastest ``tune`` value for this problem, and the timings (ms per candidate,
-    median of ``reps``).  Without ``sets`` one rb_hf_update of the frequencies ``freqs``
+    """The fastest ``tune`` value for this problem, and the timings (ms per candidate, that
+    of its form, median of ``reps``).  Without ``sets`` one rb_hf_update of the frequencies ``freqs``
     (data p_obs[len(freqs)]) is timed; with ``sets`` (index lists into ``freqs``, data
     p_obs[len(freqs)]) the whole sweep over them is, from c each time, because the
     medium the later sets see (rougher, with bent tubes) changes which choice is faster.
@@ -101,7 +107,7 @@ def tune_update(geom, c, alpha0, freqs, p_obs, prec, reps: int = 3, device=None,
     with torch.cuda.stream(stream):
         ws = rb.workspace(geom, nf, prec, dev)
         cs = torch.empty_like(c)
-        for cand in candidates(prec):
+        for cand in forms(prec):
             ms = []
             for r in range(reps + 1):
                 cs.copy_(c)
@@ -115,9 +121,11 @@ def tune_update(geom, c, alpha0, freqs, p_obs, prec, reps: int = 3, device=None,
                 if r > 0:
                     ms.append(e0.elapsed_time(e1) / len(plan))
             ms.sort()
-            times[name(cand)] = ms[len(ms) // 2]
+            for same in candidates(prec):
+                if same & 3 == cand & 3:
+                    times[name(same)] = ms[len(ms) // 2]
         del ws, cs
-    best = min(candidates(prec), key=lambda t: times[name(t)])
+    best = min(forms(prec), key=lambda t: times[name(t)])
     entry = {"tune": int(best), "choice": name(best), "ms_per_update": times,
              "timed": "sweep of %d sets" % len(plan) if sets else "one update"}
     k = key(geom, nf, prec)
