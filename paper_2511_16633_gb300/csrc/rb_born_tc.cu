@@ -193,10 +193,6 @@ constexpr uint32_t ST_ALO = 4096u, ST_B = 8192u;
 // V slices of the adjoint (K = 32): A hi (8 KB) + A lo (8 KB) + W (n rows x 32, <= 16 KB)
 constexpr uint32_t ST_VALO = 8192u, ST_VB = 16384u;
 
-__device__ __forceinline__ uint32_t pack2(__nv_bfloat16 a, __nv_bfloat16 b) {
-    return (uint32_t)__bfloat16_as_ushort(a) | ((uint32_t)__bfloat16_as_ushort(b) << 16);
-}
-
 // The two bf16 halves of a packed word, hi + lo parts added (exact: lo is below hi's ulp).
 __device__ __forceinline__ float sum_lo16(uint32_t h, uint32_t l) {
     return __uint_as_float(h << 16) + __uint_as_float(l << 16);
@@ -582,8 +578,8 @@ __global__ void __launch_bounds__(NTHR_A, 1) k_adjoint_tc(const __grid_constant_
                                 const int e0 = 8 * c + 2 * i, e1 = e0 + 1;
                                 tc::split_bf16(x[e0] * x[e0] + y[e0] * y[e0], a, al);
                                 tc::split_bf16(x[e1] * x[e1] + y[e1] * y[e1], b, bl);
-                                vh[i] = pack2(a, b);
-                                vl[i] = pack2(al, bl);
+                                vh[i] = bf16_pack2(a, b);
+                                vl[i] = bf16_pack2(al, bl);
                             }
                             *(uint4*)(vs + 64 * c) = make_uint4(vh[0], vh[1], vh[2], vh[3]);
                             *(uint4*)(vs + 64 * c + TP * 32) = make_uint4(vl[0], vl[1], vl[2], vl[3]);
@@ -1067,8 +1063,8 @@ __global__ void __launch_bounds__(NTHR_F, 1) k_forward_tc(const __grid_constant_
                     __nv_bfloat16 h0, l0, h1, l1;
                     tc::split_bf16(sum_lo16(hw[t], lw[t]) * mm, h0, l0);
                     tc::split_bf16(sum_hi16(hw[t], lw[t]) * mm, h1, l1);
-                    oh[t] = pack2(h0, h1);
-                    ol[t] = pack2(l0, l1);
+                    oh[t] = bf16_pack2(h0, h1);
+                    ol[t] = bf16_pack2(l0, l1);
                 }
                 *(uint4*)(st + aoff + 2048u * x) = make_uint4(oh[0], oh[1], oh[2], oh[3]);
                 *(uint4*)(st + ST_ALO + aoff + 2048u * x) = make_uint4(ol[0], ol[1], ol[2], ol[3]);

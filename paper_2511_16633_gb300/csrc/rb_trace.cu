@@ -415,98 +415,92 @@ __global__ void __launch_bounds__(128, 4) k_trace(GeoDev G, const float4* __rest
     };
 
     for (int k = 1; alive && k <= G.max_steps; ++k) {
-        if (alive) {
-            // direction relative to the anchor angle tha (cos / sin exact there); the
-            // anchor follows the ray whenever it has turned by more than 0.05 rad
-            // a loop rather than an if: the compiler keeps it a branch instead of evaluating
-            // the refresh on every step (it runs at most once)
-            while (fabsf(thh - tha) > 0.05f) {
-                tha = thh;
-                ray_sincos(tha, &Sa, &Ca);
-            }
-            const float dth = (thh - tha) + thl;
-            if (PUT) put_current();
-            const Deriv inc = rk4_step<INSIDE>(G, cells, cc, xh, xl, yh, yl, Ca, Sa, tha, dth, q, p);
-            const float ix = inc.x, iy = inc.y, ith = inc.th, it = inc.t, iq = inc.q, ip = inc.p, il = inc.l;
-            float nxh = xh, nxl = xl, nyh = yh, nyl = yl, nthh = thh, nthl = thl;
-            comp_add(nxh, nxl, ix);
-            comp_add(nyh, nyl, iy);
-            comp_add(nthh, nthl, ith);
-            const float nq = q + iq, np = p + ip, nl = l + il;
-            // exit test: float screen, then double decision
-            const float fx = nxh + nxl, fy = nyh + nyl;
-            bool out = false;
-            if (fx * fx + fy * fy >= G.R2 * (1.0f - 4e-6f)) out = outside_ring(nxh, nxl, nyh, nyl, G.R_d);
-            if (out) {
-                const double ax = (double)xh + (double)xl, ay = (double)yh + (double)yl;
-                const double bx = (double)nxh + (double)nxl, by = (double)nyh + (double)nyl;
-                const double lam = exit_lambda(ax, ay, bx, by, G.R_d);
-                const float lf = (float)lam;
-                const double ex = ax + lam * (bx - ax), ey = ay + lam * (by - ay);
-                const double tt = (double)trh + (double)trl;
-                const double et = __fma_rn(lam, (double)it, tt);
-                const double eth = ((double)thh + (double)thl) + lam * (((double)nthh + (double)nthl) - ((double)thh + (double)thl));
-                const float eq = q + lf * (nq - q), ep = p + lf * (np - p), el = l + lf * (nl - l);
-                const int ek = kap + ((k >= 2 && signbit(eq) != signbit(q)) ? 1 : 0);
-                const DF exd = df_from_double(ex), eyd = df_from_double(ey);
-                xh = exd.hi; xl = exd.lo; yh = eyd.hi; yl = eyd.lo;
-                const DF etd = df_from_double(et);
-                q = eq; p = ep; l = el; kap = ek; trh = etd.hi; trl = etd.lo;
+        // direction relative to the anchor angle tha (cos / sin exact there); the
+        // anchor follows the ray whenever it has turned by more than 0.05 rad
+        // a loop rather than an if: the compiler keeps it a branch instead of evaluating
+        // the refresh on every step (it runs at most once)
+        while (fabsf(thh - tha) > 0.05f) {
+            tha = thh;
+            ray_sincos(tha, &Sa, &Ca);
+        }
+        const float dth = (thh - tha) + thl;
+        if (PUT) put_current();
+        const Deriv inc = rk4_step<INSIDE>(G, cells, cc, xh, xl, yh, yl, Ca, Sa, tha, dth, q, p);
+        const float ix = inc.x, iy = inc.y, ith = inc.th, it = inc.t, iq = inc.q, ip = inc.p, il = inc.l;
+        float nxh = xh, nxl = xl, nyh = yh, nyl = yl, nthh = thh, nthl = thl;
+        comp_add(nxh, nxl, ix);
+        comp_add(nyh, nyl, iy);
+        comp_add(nthh, nthl, ith);
+        const float nq = q + iq, np = p + ip, nl = l + il;
+        // exit test: float screen, then double decision
+        const float fx = nxh + nxl, fy = nyh + nyl;
+        bool out = false;
+        if (fx * fx + fy * fy >= G.R2 * (1.0f - 4e-6f)) out = outside_ring(nxh, nxl, nyh, nyl, G.R_d);
+        if (out) {
+            const double ax = (double)xh + (double)xl, ay = (double)yh + (double)yl;
+            const double bx = (double)nxh + (double)nxl, by = (double)nyh + (double)nyl;
+            const double lam = exit_lambda(ax, ay, bx, by, G.R_d);
+            const float lf = (float)lam;
+            const double ex = ax + lam * (bx - ax), ey = ay + lam * (by - ay);
+            const double tt = (double)trh + (double)trl;
+            const double et = __fma_rn(lam, (double)it, tt);
+            const double eth = ((double)thh + (double)thl) + lam * (((double)nthh + (double)nthl) - ((double)thh + (double)thl));
+            const float eq = q + lf * (nq - q), ep = p + lf * (np - p), el = l + lf * (nl - l);
+            const int ek = kap + ((k >= 2 && signbit(eq) != signbit(q)) ? 1 : 0);
+            const DF exd = df_from_double(ex), eyd = df_from_double(ey);
+            xh = exd.hi; xl = exd.lo; yh = eyd.hi; yl = eyd.lo;
+            const DF etd = df_from_double(et);
+            q = eq; p = ep; l = el; kap = ek; trh = etd.hi; trl = etd.lo;
+            alive = false;
+            const double ddx = ex - xs_d, ddy = ey - ys_d;
+            rb_ray_end e;
+            e.t = et;
+            e.t_res = __fma_rn(-sqrt(__fma_rn(ddx, ddx, __dmul_rn(ddy, ddy))), 1.0 / G.c_ref_d, et);
+            e.x = ex;
+            e.y = ey;
+            e.theta = (float)eth;
+            e.q = eq;
+            e.p = ep;
+            e.l = el;
+            e.kappa = ek;
+            e.n_vert = k + 1;
+            ends[(size_t)t * G.n_rays + i] = e;
+            if (fan_len) atomicMax(fan_len + t, (uint32_t)(k + 1));
+        } else {
+            if (k >= 2 && signbit(nq) != signbit(q)) ++kap;
+            xh = nxh; xl = nxl; yh = nyh; yl = nyl; thh = nthh; thl = nthl;
+            comp_add(trh, trl, it);
+            q = nq; p = np; l = nl;
+            if (k == G.max_steps) {
                 alive = false;
-                {
-                    const double ddx = ex - xs_d, ddy = ey - ys_d;
-                    rb_ray_end e;
-                    e.t = et;
-                    e.t_res = __fma_rn(-sqrt(__fma_rn(ddx, ddx, __dmul_rn(ddy, ddy))), 1.0 / G.c_ref_d, et);
-                    e.x = ex;
-                    e.y = ey;
-                    e.theta = (float)eth;
-                    e.q = eq;
-                    e.p = ep;
-                    e.l = el;
-                    e.kappa = ek;
-                    e.n_vert = k + 1;
-                    ends[(size_t)t * G.n_rays + i] = e;
-                    if (fan_len) atomicMax(fan_len + t, (uint32_t)(k + 1));
-                }
-            } else {
-                if (k >= 2 && signbit(nq) != signbit(q)) ++kap;
-                xh = nxh; xl = nxl; yh = nyh; yl = nyl; thh = nthh; thl = nthl;
-                comp_add(trh, trl, it);
-                q = nq; p = np; l = nl;
-                if (k == G.max_steps) {
-                    alive = false;
-                    {
-                        const double ex = (double)xh + (double)xl, ey = (double)yh + (double)yl;
-                        const double ddx = ex - xs_d, ddy = ey - ys_d;
-                        rb_ray_end e;
-                        const double tt = (double)trh + (double)trl;
-                        e.t = tt;
-                        e.t_res = tt - sqrt(ddx * ddx + ddy * ddy) * (1.0 / G.c_ref_d);
-                        e.x = ex;
-                        e.y = ey;
-                        e.theta = thh + thl;
-                        e.q = q;
-                        e.p = p;
-                        e.l = l;
-                        e.kappa = kap;
-                        e.n_vert = -1;
-                        ends[(size_t)t * G.n_rays + i] = e;
-                        atomicAdd(counters + CNT_LOST, 1u);
-                        if (fan_len) atomicMax(fan_len + t, (uint32_t)(G.max_steps + 1));
-                    }
-                }
+                const double ex = (double)xh + (double)xl, ey = (double)yh + (double)yl;
+                const double ddx = ex - xs_d, ddy = ey - ys_d;
+                rb_ray_end e;
+                const double tt = (double)trh + (double)trl;
+                e.t = tt;
+                e.t_res = tt - sqrt(ddx * ddx + ddy * ddy) * (1.0 / G.c_ref_d);
+                e.x = ex;
+                e.y = ey;
+                e.theta = thh + thl;
+                e.q = q;
+                e.p = p;
+                e.l = l;
+                e.kappa = kap;
+                e.n_vert = -1;
+                ends[(size_t)t * G.n_rays + i] = e;
+                atomicAdd(counters + CNT_LOST, 1u);
+                if (fan_len) atomicMax(fan_len + t, (uint32_t)(G.max_steps + 1));
             }
-            if (SAMPLES) {
-                const size_t o = sbase + (size_t)k;
-                const double vx = (double)xh + (double)xl, vy = (double)yh + (double)yl;
-                S.vx[o] = (float)vx;
-                S.vy[o] = (float)vy;
-                S.vt[o] = (double)trh + (double)trl;
-                S.vq[o] = q;
-                S.vl[o] = l;
-                S.vkappa[o] = kap;
-            }
+        }
+        if (SAMPLES) {
+            const size_t o = sbase + (size_t)k;
+            const double vx = (double)xh + (double)xl, vy = (double)yh + (double)yl;
+            S.vx[o] = (float)vx;
+            S.vy[o] = (float)vy;
+            S.vt[o] = (double)trh + (double)trl;
+            S.vq[o] = q;
+            S.vl[o] = l;
+            S.vkappa[o] = kap;
         }
     }
     if (PUT) put_current();
