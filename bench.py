@@ -138,7 +138,7 @@ def adjoint_issue_ratio(n):
 # set to None whenever the kernel changes until it is captured again.
 ADJ_TRAFFIC_BYTES = 2150002944 + 469237248
 ADJ_TRAFFIC_SOURCE = ("ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum, one k_adjoint_tc launch on "
-                      "breast512 (profiles/launches_breast512_bf16x3.md)")
+                      "breast512, kernel as of commit 862c275 (profiles/launches_breast512_bf16x3.md)")
 
 
 def rays_grid_bytes(cfg, n_vertices):

@@ -1107,8 +1107,11 @@ __global__ void __launch_bounds__(NTHR_F, 1) k_forward_tc(const __grid_constant_
 // a computed block (right of its row block's first column), so entry (e, r), e <= r, is
 // read row-wise and written to d[e][r] and d[r][e].  YS warps take 32 consecutive r of one e:
 // each every YS-th split, the first adds the warps' sums in order.  YS = 1 where the
-// entries alone fill the chip (256 elements: 12 us for 52 splits; eight warps an entry, with
-// their barriers, 43), 8 below 128 elements (64: 27 us by single warps, 152 splits each).
+// entries alone fill the chip (128 to 512 elements at 511 x 389 pixels: 8 to 12 us; eight warps
+// an entry, with their barriers, 43 for 256), 8 below 128 elements (64: 5 us; by single warps
+// of 152 splits each, with one load under way, 27).  Loads go out eight splits ahead: left to the
+// compiler, the loop of calls that write d waited for every split (256 elements, 48 splits: 45 us
+// against 8).
 template <int YS>
 __global__ void __launch_bounds__(256) k_forward_tc_reduce(FwdArgs A, float2* __restrict__ d_out, const uint8_t* __restrict__ w,
                                                            double* __restrict__ den_part) {

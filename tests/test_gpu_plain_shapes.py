@@ -33,9 +33,9 @@ def test_adjoint_of_small_rings(dev, n, nx, ny):  # noqa: F811
             assert _rel(h, w2 * w2 * (P * (W.double() @ P)).sum(0)) <= 1e-5
 
 
-# two chunks (the smallest grid that a ring fits), eight, ten, and the fixed scratch's single chunk
-# for a thousand elements
-@pytest.mark.parametrize("n,nx,ny", [(70, 6, 6), (33, 16, 16), (70, 17, 17), (600, 16, 15), (1000, 12, 11)])
+# two chunks (on the coarsest grid whose h / 4, the floor of |q|, lies below the tables' q), eight,
+# ten, and the fixed scratch's single chunk for a thousand elements
+@pytest.mark.parametrize("n,nx,ny", [(70, 7, 7), (33, 16, 16), (70, 17, 17), (600, 16, 15), (1000, 12, 11)])
 def test_forward_of_few_chunks(dev, n, nx, ny):  # noqa: F811
     geom, tab, c, G, f, g = _problem(dev, n, nx, ny)
     m = 1e-9 * torch.randn(nx * ny, generator=g, device=dev)
